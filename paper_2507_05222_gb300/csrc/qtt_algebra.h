@@ -111,6 +111,5 @@ void cg_tc(Ctx& c, const double* L, const double* W, const double* R, const doub
 void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev);
 void sqrt_dev(Ctx& c, const double* in, double* out);
 qtt_mps* encode_dense(Ctx& c, const double* dense_dev, int n, int d, int chi, double eps);
-void decode_dense(Ctx& c, const qtt_mps* x, double* dense_dev);
 
 }  // namespace qtt

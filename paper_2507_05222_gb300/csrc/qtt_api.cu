@@ -448,10 +448,10 @@ int qtt_decode(qtt_ctx* ctx, const qtt_mps* x, double* dense, int kind) {
   int64_t N = 1;
   for (int i = 0; i < x->n; ++i) N *= x->d;
   if (kind == QTT_DEVICE) {
-    decode_dense(c, x, dense);
+    decode_mid(c, x, dense);
   } else {
     DBuf buf(&c, size_t(N));
-    decode_dense(c, x, buf.p);
+    decode_mid(c, x, buf.p);
     QTT_CUDA(cudaMemcpyAsync(dense, buf.p, N * sizeof(double), kind_out(kind), c.stream));
     QTT_CUDA(cudaStreamSynchronize(c.stream));
   }
