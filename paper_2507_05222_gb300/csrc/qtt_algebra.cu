@@ -480,6 +480,13 @@ struct CutProj {
   bool trans = false;
 };
 
+// Eigenpairs of a cut's density matrix S (positive semidefinite; S = F^T F when F is given).
+static void density_eigh(Ctx& c, int n, const double* S, double* w, double* V, int keep, const double* F = nullptr,
+                         int m = 0) {
+  if (eigh_psd_fits(n, m)) eigh_psd(c, n, S, w, V, keep, F, m);
+  else eigh(c, n, S, w, V, keep, F, m);
+}
+
 qtt_mps* round_gram(Ctx& c, const qtt_mps* y, int chi, double eps) {
   const int n = y->n, d = y->d;
   const std::vector<int>& R = y->bonds;
@@ -553,7 +560,7 @@ qtt_mps* round_gram(Ctx& c, const qtt_mps* y, int chi, double eps) {
       DBuf T1(&c, size_t(a0) * nv), rho(&c, size_t(nv) * nv), w(&c, size_t(nv)), V(&c, size_t(nv) * nv);
       einsum(c, "aA,asc->Asc", 1.0, tv(G[k].p, {a0, a0}), tv(Z.p, {a0, d, c1}), 0.0, tv(T1.p, {a0, d, c1}));
       einsum(c, "Asc,AtD->sctD", 1.0, tv(T1.p, {a0, d, c1}), tv(Z.p, {a0, d, c1}), 0.0, tv(rho.p, {d, c1, d, c1}));
-      eigh(c, nv, rho.p, w.p, V.p, std::min(std::min(chi, m[k]), nv));
+      density_eigh(c, nv, rho.p, w.p, V.p, std::min(std::min(chi, m[k]), nv));
       int bk = choose_rank(c, w.p, nv, chi, eps, std::min(m[k], nv));
       add_discarded(c, rho.p, w.p, nv, bk);
       if (!z) out[k].reset(&c, size_t(bk) * nv);
@@ -699,7 +706,7 @@ qtt_mps* apply_round_gram(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi, d
            tv(T2.p, {w0, a0, d, c1}));
     einsum(c, "WAsc,WASC->scSC", 1.0, tv(T2.p, {w0, a0, d, c1}), tv(Z.p, {w0, a0, d, c1}), 0.0,
            tv(rho.p, {d, c1, d, c1}));
-    eigh(c, nv, rho.p, wv.p, V.p, bk);
+    density_eigh(c, nv, rho.p, wv.p, V.p, bk);
     add_discarded(c, rho.p, wv.p, nv, bk);
     top_vectors_as_core(c, V.p, nv, bk, z->core(k));
     DBuf Pn(&c, size_t(wa) * bk);
@@ -840,7 +847,7 @@ qtt_mps* apply_round_sketch(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi,
     gemm(c, 1, r, nv, wa, 1.0, F[k - 1].p, 0, wa, 1, Z.p, 0, nv, 1, 0.0, A.p, 0, nv, 1);
     F[k - 1] = DBuf();
     gemm(c, 1, nv, nv, r, 1.0, A.p, 0, 1, nv, A.p, 0, nv, 1, 0.0, S.p, 0, nv, 1);
-    eigh(c, nv, S.p, wv.p, V.p, bk, A.p, r);
+    density_eigh(c, nv, S.p, wv.p, V.p, bk, A.p, r);
     if (c.disc_acc && bk < nv) {
       k_disc_add_tail<<<1, 1, 0, c.stream>>>(wv.p, nv, bk, c.disc_acc);
       after_launch(c, "disc_add_tail");
@@ -1136,7 +1143,7 @@ qtt_mps* zipup_hadamard(Ctx& c, const qtt_mps* a, const qtt_mps* b, int chi) {
     }
     DBuf rho(&c, size_t(nv) * nv), w(&c, size_t(nv)), V(&c, size_t(nv) * nv);
     gemm(c, 1, nv, nv, ab, 1.0, T.p, 0, 1, nv, T.p, 0, nv, 1, 0.0, rho.p, 0, nv, 1);
-    eigh(c, nv, rho.p, w.p, V.p, bk);
+    density_eigh(c, nv, rho.p, w.p, V.p, bk);
     top_vectors_as_core(c, V.p, nv, bk, out[k].p);
     // C_new(beta, a, b) = sum_{s,c} T(a, b, s, c) V(sc, beta)
     gemm(c, 1, bk, ab, nv, 1.0, V.p, 0, 1, nv, T.p, 0, 1, nv, 0.0, Cn.p, 0, ab, 1);
@@ -1204,7 +1211,7 @@ qtt_mps* encode_dense(Ctx& c, const double* dense_dev, int n, int d, int chi, do
     }
     DBuf rho(&c, size_t(nv) * nv), w(&c, size_t(nv)), V(&c, size_t(nv) * nv);
     gemm(c, 1, nv, nv, rows, 1.0, cur, 0, 1, nv, cur, 0, nv, 1, 0.0, rho.p, 0, nv, 1);
-    eigh(c, nv, rho.p, w.p, V.p, bk);
+    density_eigh(c, nv, rho.p, w.p, V.p, bk);
     add_discarded(c, rho.p, w.p, nv, bk);
     top_vectors_as_core(c, V.p, nv, bk, z->core(k));
     DBuf nxt(&c, size_t(rows) * bk);

