@@ -24,129 +24,248 @@ constexpr float NN_B1 = 0.9f, NN_B2 = 0.999f, NN_EPS = 1e-8f;
 
 unsigned nn_blocks(int64_t n, int t) { return unsigned(std::min<int64_t>((n + t - 1) / t, 65535 * 8)); }
 
-// input affine (x - shift[c]) * scale[c] applied on load when shift/scale are given (layer 0)
-__global__ void k_conv_fwd(int B, int ci, int co, int H, int W, const float* __restrict__ x,
-                           const float* __restrict__ shift, const float* __restrict__ scale,
-                           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ y, int relu) {
-  const int64_t total = int64_t(B) * co * H * W;
-  for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < total;
-       idx += int64_t(gridDim.x) * blockDim.x) {
-    const int j = int(idx % W);
-    const int i = int((idx / W) % H);
-    const int o = int((idx / (int64_t(W) * H)) % co);
-    const int n = int(idx / (int64_t(W) * H * co));
-    float s = b[o];
-    for (int c = 0; c < ci; ++c) {
-      const float sh = shift ? shift[c] : 0.f, sc = scale ? scale[c] : 1.f;
-      const float* xc = x + (int64_t(n) * ci + c) * H * W;
-      const float* wc = w + (int64_t(o) * ci + c) * 9;
+// The convolution and its data gradient.  FLIP = false: out[n, o] = b[o] + sum_c w[o, c] * in[n, c]
+// (with ReLU, and the layer's input affine (x - shift[c]) scale[c], zero outside the grid in the
+// mapped values); FLIP = true: out[n, c] = sum_o w[o, c] (transposed stencil) in[n, o], zero where
+// the activation `act` of the layer below is not positive (its ReLU).  A CTA computes an R x 32
+// tile of pixels for 4 COT channels: a thread has four neighbouring pixels of COT channels in
+// registers, input rows and weights staged in shared memory CC input channels at a time, so that
+// 36 COT multiply-adds take 18 + 9 COT / 4 shared loads: the FP32 pipe bounds it, where one thread
+// per output loaded an input and a weight for each multiply-add.  The order of each output's sum is
+// unchanged (input channels, then taps).  With k_conv_wgrad a training step of 8 x 128 x 128 cells,
+// width 32, depth 4 (15 GFLOP) went from 14.4 to 1.02 ms.
+template <int COT, bool FLIP>
+__global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, const float* __restrict__ in,
+                                              const float* __restrict__ shift, const float* __restrict__ scale,
+                                              const float* __restrict__ w, const float* __restrict__ b,
+                                              const float* __restrict__ act, float* __restrict__ out, int relu) {
+  constexpr int CC = 4;                          // input channels per stage
+  constexpr int NG = COT == 1 ? 1 : 4;           // channel groups of a CTA
+  constexpr int R = 256 / NG / 8;                // tile rows (8 threads of four pixels a row)
+  constexpr int CO = COT * NG;
+  __shared__ float xs[CC][R + 2][36];
+  __shared__ __align__(16) float ws[CC][9][CO];
+  const int tid = threadIdx.x;
+  const int px = tid & 7, py = (tid >> 3) % R, og = tid / (8 * R);
+  const int tw = (W + 31) / 32, th = (H + R - 1) / R;
+  const int n = blockIdx.x / (tw * th), t = blockIdx.x % (tw * th);
+  const int i0 = (t / tw) * R, j0 = (t % tw) * 32, o0 = blockIdx.y * CO;
+  const int64_t per = int64_t(H) * W;
+  float acc[COT][4];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int ii = i + a - 1;
-        if (ii < 0 || ii >= H) continue;
+  for (int o = 0; o < COT; ++o) {
+    const int oo = o0 + og * COT + o;
+    const float bv = (!FLIP && oo < no) ? b[oo] : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[o][q] = bv;
+  }
+  for (int c0 = 0; c0 < ni; c0 += CC) {
+    __syncthreads();
+    for (int e = tid; e < CC * (R + 2) * 34; e += 256) {
+      const int c = e / ((R + 2) * 34), r = (e / 34) % (R + 2), q = e % 34;
+      const int ii = i0 + r - 1, ch = c0 + c;
+      int jj = j0 + q - 1;
+      jj = jj < 0 ? jj + W : jj;
+      while (jj >= W) jj -= W;                   // periodic; columns beyond the grid are not written out
+      float v = 0.f;
+      if (ch < ni && ii >= 0 && ii < H) {
+        v = in[(int64_t(n) * ni + ch) * per + int64_t(ii) * W + jj];
+        if (!FLIP && shift) v = (v - shift[ch]) * scale[ch];
+      }
+      xs[c][r][q] = v;
+    }
+    for (int e = tid; e < CC * 9 * CO; e += 256) {
+      const int c = e / (9 * CO), k = (e / CO) % 9, o = e % CO;
+      const int ch = c0 + c, oo = o0 + o;
+      float v = 0.f;
+      if (ch < ni && oo < no) v = FLIP ? w[(int64_t(ch) * no + oo) * 9 + k] : w[(int64_t(oo) * ni + ch) * 9 + k];
+      ws[c][k][o] = v;
+    }
+    __syncthreads();
+    const int nc = min(CC, ni - c0);
+    for (int c = 0; c < nc; ++c) {
+      float x[3][6];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) x[a][q] = xs[c][py + a][4 * px + q];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
-          int jj = j + e - 1;
-          jj = jj < 0 ? jj + W : (jj >= W ? jj - W : jj);
-          s = fmaf(wc[a * 3 + e], (xc[int64_t(ii) * W + jj] - sh) * sc, s);
+          const int ra = FLIP ? 2 - a : a, re = FLIP ? 2 - e : e;
+          if (COT == 1) {
+            const float wv = ws[c][a * 3 + e][og];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[0][q] = fmaf(wv, x[ra][q + re], acc[0][q]);
+          } else {
+#pragma unroll
+            for (int o = 0; o < COT; o += 4) {
+              const float4 wv = *reinterpret_cast<const float4*>(&ws[c][a * 3 + e][og * COT + o]);
+              const float wq[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[(o + u) % COT][q] = fmaf(wq[u], x[ra][q + re], acc[(o + u) % COT][q]);
+            }
+          }
         }
-      }
     }
-    y[idx] = relu ? fmaxf(s, 0.f) : s;
+  }
+  const int i = i0 + py;
+  if (i >= H) return;
+#pragma unroll
+  for (int o = 0; o < COT; ++o) {
+    const int oo = o0 + og * COT + o;
+    if (oo >= no) continue;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + 4 * px + q;
+      if (j >= W) continue;
+      const int64_t g = (int64_t(n) * no + oo) * per + int64_t(i) * W + j;
+      float v = acc[o][q];
+      if (FLIP) v = act[g] > 0.f ? v : 0.f;
+      else if (relu) v = fmaxf(v, 0.f);
+      out[g] = v;
+    }
   }
 }
 
-// dx[n, c, i, j] = sum_{o, a, e} w[o, c, a, e] dy[n, o, i - a + 1, j - e + 1]
-__global__ void k_conv_bwd_data(int B, int ci, int co, int H, int W, const float* __restrict__ dy,
-                                const float* __restrict__ w, float* __restrict__ dx) {
-  const int64_t total = int64_t(B) * ci * H * W;
-  for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < total;
-       idx += int64_t(gridDim.x) * blockDim.x) {
-    const int j = int(idx % W);
-    const int i = int((idx / W) % H);
-    const int c = int((idx / (int64_t(W) * H)) % ci);
-    const int n = int(idx / (int64_t(W) * H * ci));
-    float s = 0.f;
-    for (int o = 0; o < co; ++o) {
-      const float* dyo = dy + (int64_t(n) * co + o) * H * W;
-      const float* wo = w + (int64_t(o) * ci + c) * 9;
+// Weight and bias gradients: part[g][(o ci + c) 9 + tap] and part[g][co ci 9 + o] = the sums over the
+// pixel tiles g, g + gridDim.x, ... of dy[n, o, i, j] x'[n, c, i + a - 1, j + e - 1] (x' with the
+// layer's input affine) and of dy.  A CTA keeps a chunk of 32 x 32 channel pairs: a thread has the
+// nine taps of 4 x 2 of them (72 sums) in registers and slides a 3 x 3 window along the rows of a
+// 4 x 32 tile staged in shared memory; where the layer has fewer channels the threads share the
+// tile's rows instead (pg).  The partial sums are added by k_conv_wsum in a fixed order.  (One CTA
+// per weight reads both activations from L2 for every one of the 9 co ci weights.)
+constexpr int CW_TR = 4, CW_TC = 32, CW_CH = 32, CW_XS = 34, CW_YS = 36;
+__global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H, int W, const float* __restrict__ x,
+                                                    const float* __restrict__ shift, const float* __restrict__ scale,
+                                                    const float* __restrict__ dy, float* __restrict__ part) {
+  extern __shared__ __align__(16) float cw_sm[];
+  float* xs = cw_sm;                                          // [(TR + 2)][TC + 2][CW_XS]
+  float* ys = xs + (CW_TR + 2) * (CW_TC + 2) * CW_XS;         // [TR][TC][CW_YS]
+  const int tid = threadIdx.x;
+  const int o0 = (blockIdx.y % ((co + CW_CH - 1) / CW_CH)) * CW_CH, c0 = (blockIdx.y / ((co + CW_CH - 1) / CW_CH)) * CW_CH;
+  const int no = min(CW_CH, co - o0), nc = min(CW_CH, ci - c0);
+  const int OG = (no + 3) / 4, CG = (nc + 1) / 2, PG = min(CW_TR, 256 / (OG * CG));
+  const int og = tid % OG, cg = (tid / OG) % CG, pg = tid / (OG * CG);
+  const int64_t per = int64_t(H) * W;
+  const int tw = (W + CW_TC - 1) / CW_TC, th = (H + CW_TR - 1) / CW_TR, ntiles = B * tw * th;
+  float acc[4][2][9], bs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int ii = i - a + 1;
-        if (ii < 0 || ii >= H) continue;
+  for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          int jj = j - e + 1;
-          jj = jj < 0 ? jj + W : (jj >= W ? jj - W : jj);
-          s = fmaf(wo[a * 3 + e], dyo[int64_t(ii) * W + jj], s);
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) acc[o][c][k] = 0.f;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int n = t / (tw * th), i0 = ((t / tw) % th) * CW_TR, j0 = (t % tw) * CW_TC;
+    __syncthreads();
+    for (int e = tid; e < CW_CH * (CW_TR + 2) * (CW_TC + 2); e += 256) {
+      const int q = e % (CW_TC + 2), r = (e / (CW_TC + 2)) % (CW_TR + 2), c = e / ((CW_TC + 2) * (CW_TR + 2));
+      const int ii = i0 + r - 1;
+      int jj = j0 + q - 1;
+      jj = jj < 0 ? jj + W : jj;
+      while (jj >= W) jj -= W;
+      float v = 0.f;
+      if (c < nc && ii >= 0 && ii < H) {
+        v = x[(int64_t(n) * ci + c0 + c) * per + int64_t(ii) * W + jj];
+        if (shift) v = (v - shift[c0 + c]) * scale[c0 + c];
+      }
+      xs[(r * (CW_TC + 2) + q) * CW_XS + c] = v;
+    }
+    for (int e = tid; e < CW_CH * CW_TR * CW_TC; e += 256) {
+      const int q = e % CW_TC, r = (e / CW_TC) % CW_TR, o = e / (CW_TC * CW_TR);
+      const int ii = i0 + r, jj = j0 + q;
+      ys[(r * CW_TC + q) * CW_YS + o] =
+          (o < no && ii < H && jj < W) ? dy[(int64_t(n) * co + o0 + o) * per + int64_t(ii) * W + jj] : 0.f;
+    }
+    __syncthreads();
+    if (pg < PG) {
+      for (int r = pg; r < CW_TR; r += PG) {
+        float2 win[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            win[a][e + 1] = *reinterpret_cast<const float2*>(&xs[((r + a) * (CW_TC + 2) + e) * CW_XS + 2 * cg]);
+#pragma unroll 4
+        for (int q = 0; q < CW_TC; ++q) {
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            win[a][0] = win[a][1];
+            win[a][1] = win[a][2];
+            win[a][2] = *reinterpret_cast<const float2*>(&xs[((r + a) * (CW_TC + 2) + q + 2) * CW_XS + 2 * cg]);
+          }
+          const float4 g4 = *reinterpret_cast<const float4*>(&ys[(r * CW_TC + q) * CW_YS + 4 * og]);
+          const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            if (cg == 0) bs[o] += g[o];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+              for (int e = 0; e < 3; ++e) {
+                acc[o][0][3 * a + e] = fmaf(g[o], win[a][e].x, acc[o][0][3 * a + e]);
+                acc[o][1][3 * a + e] = fmaf(g[o], win[a][e].y, acc[o][1][3 * a + e]);
+              }
+          }
         }
       }
     }
-    dx[idx] = s;
   }
-}
-
-// One block per weight (o, c, a, e) -- blocks [0, co ci 9) -- and per bias o -- blocks
-// [co ci 9, co ci 9 + co): dw = sum_{n, i, j} dy[n, o, i, j] x'[n, c, i + a - 1, j + e - 1] with the
-// layer's input affine, db = sum dy[n, o, :, :].  Fixed summation order (per-thread strides,
-// then a fixed tree): deterministic.
-__global__ void k_conv_bwd_w(int B, int ci, int co, int H, int W, const float* __restrict__ x,
-                             const float* __restrict__ shift, const float* __restrict__ scale,
-                             const float* __restrict__ dy, float* __restrict__ dw, float* __restrict__ db) {
-  __shared__ float red[32];
-  const int blk = blockIdx.x;
-  const bool bias = blk >= co * ci * 9;
-  int o, c = 0, a = 0, e = 0;
-  if (bias) {
-    o = blk - co * ci * 9;
-  } else {
-    o = blk / (ci * 9);
-    const int r = blk % (ci * 9);
-    c = r / 9;
-    a = (r % 9) / 3;
-    e = r % 3;
-  }
-  const float sh = (!bias && shift) ? shift[c] : 0.f, sc = (!bias && scale) ? scale[c] : 1.f;
-  const int64_t per = int64_t(H) * W, total = int64_t(B) * per;
-  float s = 0.f;
-  for (int64_t t = threadIdx.x; t < total; t += blockDim.x) {
-    const int n = int(t / per);
-    const int i = int((t % per) / W), j = int(t % W);
-    const float g = dy[(int64_t(n) * co + o) * per + int64_t(i) * W + j];
-    if (bias) {
-      s += g;
-    } else {
-      const int ii = i + a - 1;
-      if (ii < 0 || ii >= H) continue;
-      int jj = j + e - 1;
-      jj = jj < 0 ? jj + W : (jj >= W ? jj - W : jj);
-      s = fmaf(g, (x[(int64_t(n) * ci + c) * per + int64_t(ii) * W + jj] - sh) * sc, s);
-    }
-  }
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  // the row groups' sums, in order, into shared memory, then out
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (threadIdx.x == 0) {
-      if (bias) db[o] = v;
-      else dw[blk] = v;
+  float* red = cw_sm;                                          // [32][32][9] then [32]
+  for (int p = 0; p < PG; ++p) {
+    if (pg == p) {
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int k = 0; k < 9; ++k) {
+            float* d = &red[((4 * og + o) * CW_CH + 2 * cg + c) * 9 + k];
+            *d = p == 0 ? acc[o][c][k] : *d + acc[o][c][k];
+          }
+        if (cg == 0) {
+          float* d = &red[CW_CH * CW_CH * 9 + 4 * og + o];
+          *d = p == 0 ? bs[o] : *d + bs[o];
+        }
+      }
     }
+    __syncthreads();
   }
+  float* dst = part + int64_t(blockIdx.x) * (int64_t(co) * ci * 9 + co);
+  for (int e = tid; e < no * nc * 9; e += 256) {
+    const int o = e / (nc * 9), c = (e / 9) % nc, k = e % 9;
+    dst[(int64_t(o0 + o) * ci + c0 + c) * 9 + k] = red[(o * CW_CH + c) * 9 + k];
+  }
+  if (c0 == 0)
+    for (int o = tid; o < no; o += 256) dst[int64_t(co) * ci * 9 + o0 + o] = red[CW_CH * CW_CH * 9 + o];
+}
+constexpr size_t kWgradSmem = ((CW_TR + 2) * (CW_TC + 2) * CW_XS + CW_TR * CW_TC * CW_YS) * sizeof(float);
+static_assert(kWgradSmem >= (CW_CH * CW_CH * 9 + CW_CH) * sizeof(float), "wgrad reduction buffer");
+
+// grad[e] = sum_g part[g][e], eight lanes a value (strided over g, then a fixed tree).
+__global__ void __launch_bounds__(256) k_conv_wsum(int64_t n, int G, const float* __restrict__ part, float* __restrict__ grad) {
+  const int64_t e = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 3;
+  const int l = threadIdx.x & 7;
+  float s = 0.f;
+  if (e < n)
+    for (int g = l; g < G; g += 8) s += part[int64_t(g) * n + e];
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (e < n && l == 0) grad[e] = s;
 }
 
-__global__ void k_relu_mask(int64_t n, const float* __restrict__ act, float* __restrict__ g) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    if (!(act[i] > 0.f)) g[i] = 0.f;
-}
-
-// dpred = 2 (pred - y / out_scale) / n; *loss = mean squared difference (one block, fixed order)
-__global__ void k_mse(int64_t n, const float* __restrict__ pred, const float* __restrict__ y, float inv_out,
-                      float* __restrict__ dpred, float* __restrict__ loss) {
-  __shared__ double red[32];
+// dpred = 2 (pred - y / out_scale) / n and, per block, the sum of squared differences.
+constexpr int MSE_BLOCKS = 256;
+__global__ void __launch_bounds__(256) k_mse(int64_t n, const float* __restrict__ pred, const float* __restrict__ y,
+                                             float inv_out, float* __restrict__ dpred, double* __restrict__ part) {
+  __shared__ double red[8];
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     const float d = pred[i] - y[i] * inv_out;
     dpred[i] = 2.f * d / float(n);
     s += double(d) * d;
@@ -154,11 +273,19 @@ __global__ void k_mse(int64_t n, const float* __restrict__ pred, const float* __
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (threadIdx.x == 0) *loss = float(v / double(n));
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < 8; ++w) v += red[w];
+    part[blockIdx.x] = v;
   }
+}
+
+// *loss = mean of the blocks' sums (fixed order)
+__global__ void k_mse_sum(int64_t n, int G, const double* __restrict__ part, float* __restrict__ loss) {
+  double v = 0.0;
+  for (int i = threadIdx.x; i < G; i += 32) v += part[i];
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if (threadIdx.x == 0) *loss = float(v / double(n));
 }
 
 __global__ void k_adam(int64_t n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -244,12 +371,34 @@ __global__ void k_moments(int64_t n, const float* __restrict__ x, double* __rest
   }
 }
 
+// Channels in groups of 32 (eight a thread) where the layer has more than four, else one a thread.
+template <bool FLIP>
+void conv(Ctx& c, int B, int ni, int no, int H, int W, const float* in, const float* shift, const float* scale,
+          const float* w, const float* b, const float* act, float* out, int relu) {
+  const int R = no > 4 ? 8 : 32;
+  const int64_t tiles = int64_t(B) * ((W + 31) / 32) * ((H + R - 1) / R);
+  if (no > 4)
+    k_conv<8, FLIP><<<dim3(unsigned(tiles), unsigned((no + 31) / 32)), 256, 0, c.stream>>>(ni, no, H, W, in, shift, scale,
+                                                                                          w, b, act, out, relu);
+  else
+    k_conv<1, FLIP><<<dim3(unsigned(tiles), unsigned(no)), 256, 0, c.stream>>>(ni, no, H, W, in, shift, scale, w, b, act,
+                                                                              out, relu);
+  after_launch(c, FLIP ? "nn_conv_bwd_data" : "nn_conv_fwd");
+}
+
 float* fbuf(DBuf& b, Ctx& c, int64_t nfloats) {
   b.reset(&c, size_t((nfloats + 1) / 2));
   return reinterpret_cast<float*>(b.p);
 }
 
 }  // namespace
+
+static void init_nn_attributes() {
+  static bool done = false;
+  if (done) return;
+  QTT_CUDA(cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kWgradSmem)));
+  done = true;
+}
 
 int64_t nn_param_count(int c_in, int width, int depth) {
   int64_t n = 0;
@@ -270,9 +419,14 @@ Net::Net(Ctx& c, int c_in_, int width_, int depth_, const float* params_host)
     ci_.push_back(ci);
     co_.push_back(co);
   }
-  for (float** p : {&params, &m, &v, &grad}) QTT_CUDA(cudaMalloc(p, size_t(nparam) * sizeof(float)));
-  QTT_CUDA(cudaMalloc(&shift, size_t(c_in) * sizeof(float)));
-  QTT_CUDA(cudaMalloc(&scale, size_t(c_in) * sizeof(float)));
+  // one block of the context's pool: parameters, both moments, gradient, input affine
+  const int64_t np = (nparam + 3) / 4 * 4;
+  params = fbuf(store, c, 4 * np + 2 * c_in);
+  m = params + np;
+  v = m + np;
+  grad = v + np;
+  shift = grad + np;
+  scale = shift + c_in;
   QTT_CUDA(cudaMemcpyAsync(params, params_host, size_t(nparam) * sizeof(float), cudaMemcpyHostToDevice, c.stream));
   QTT_CUDA(cudaMemsetAsync(m, 0, size_t(nparam) * sizeof(float), c.stream));
   QTT_CUDA(cudaMemsetAsync(v, 0, size_t(nparam) * sizeof(float), c.stream));
@@ -284,8 +438,6 @@ Net::Net(Ctx& c, int c_in_, int width_, int depth_, const float* params_host)
 
 Net::~Net() {
   if (ctx) cudaStreamSynchronize(ctx->stream);
-  for (float* p : {params, m, v, grad, shift, scale})
-    if (p) cudaFree(p);
 }
 
 void Net::set_scaling(const float* in_shift, const float* in_scale, float out_scale_) {
@@ -310,9 +462,8 @@ void Net::forward(int B, int H, int W, const float* x, std::vector<DBuf>& acts) 
     float* out = fbuf(acts[k], c, int64_t(B) * co * H * W);
     const float* w = params + off;
     const float* b = w + int64_t(co) * ci * 9;
-    k_conv_fwd<<<nn_blocks(int64_t(B) * co * H * W, 256), 256, 0, c.stream>>>(
-        B, ci, co, H, W, in, k == 0 ? shift : nullptr, k == 0 ? scale : nullptr, w, b, out, k < depth - 1 ? 1 : 0);
-    after_launch(c, "nn_conv_fwd");
+    conv<false>(c, B, ci, co, H, W, in, k == 0 ? shift : nullptr, k == 0 ? scale : nullptr, w, b, nullptr, out,
+                k < depth - 1 ? 1 : 0);
     off += int64_t(co) * ci * 9 + co;
     in = out;
   }
@@ -336,9 +487,14 @@ float Net::train_step(int B, int H, int W, const float* x, const float* y, float
   const int64_t per = int64_t(H) * W;
   DBuf dyb, dxb;
   float* dy = fbuf(dyb, c, int64_t(B) * per);
-  k_mse<<<1, 1024, 0, c.stream>>>(int64_t(B) * per, reinterpret_cast<float*>(acts[depth - 1].p), y,
-                                  1.f / out_scale, dy, loss_dev);
+  DBuf mpart(&c, MSE_BLOCKS);
+  const int mg = int(std::min<int64_t>(MSE_BLOCKS, (int64_t(B) * per + 255) / 256));
+  k_mse<<<mg, 256, 0, c.stream>>>(int64_t(B) * per, reinterpret_cast<float*>(acts[depth - 1].p), y, 1.f / out_scale, dy,
+                                  mpart.p);
   after_launch(c, "nn_mse");
+  k_mse_sum<<<1, 32, 0, c.stream>>>(int64_t(B) * per, mg, mpart.p, loss_dev);
+  after_launch(c, "nn_mse_sum");
+  init_nn_attributes();
   // parameter offsets per layer
   std::vector<int64_t> offs(depth);
   int64_t off = 0;
@@ -350,18 +506,21 @@ float Net::train_step(int B, int H, int W, const float* x, const float* y, float
     const int ci = ci_[k], co = co_[k];
     const float* in = k == 0 ? x : reinterpret_cast<float*>(acts[k - 1].p);
     float* dw = grad + offs[k];
-    float* db = dw + int64_t(co) * ci * 9;
-    k_conv_bwd_w<<<unsigned(co * ci * 9 + co), 256, 0, c.stream>>>(B, ci, co, H, W, in, k == 0 ? shift : nullptr,
-                                                                   k == 0 ? scale : nullptr, dy, dw, db);
-    after_launch(c, "nn_conv_bwd_w");
+    const int64_t nw = int64_t(co) * ci * 9 + co;
+    const int64_t tiles = int64_t(B) * ((W + CW_TC - 1) / CW_TC) * ((H + CW_TR - 1) / CW_TR);
+    const int chunks = ((co + CW_CH - 1) / CW_CH) * ((ci + CW_CH - 1) / CW_CH);
+    const int G = int(std::min<int64_t>(tiles, std::max(1, 2 * c.num_sms / chunks)));   // two CTAs per SM
+    DBuf wpart;
+    float* wp = fbuf(wpart, c, nw * G);
+    k_conv_wgrad<<<dim3(unsigned(G), unsigned(chunks)), 256, kWgradSmem, c.stream>>>(
+        B, ci, co, H, W, in, k == 0 ? shift : nullptr, k == 0 ? scale : nullptr, dy, wp);
+    after_launch(c, "nn_conv_wgrad");
+    k_conv_wsum<<<unsigned((nw * 8 + 255) / 256), 256, 0, c.stream>>>(nw, G, wp, dw);
+    after_launch(c, "nn_conv_wsum");
     if (k > 0) {
       float* dx = fbuf(dxb, c, int64_t(B) * ci * per);
-      k_conv_bwd_data<<<nn_blocks(int64_t(B) * ci * per, 256), 256, 0, c.stream>>>(B, ci, co, H, W, dy,
-                                                                                  params + offs[k], dx);
-      after_launch(c, "nn_conv_bwd_data");
-      k_relu_mask<<<nn_blocks(int64_t(B) * ci * per, 256), 256, 0, c.stream>>>(
-          int64_t(B) * ci * per, reinterpret_cast<float*>(acts[k - 1].p), dx);
-      after_launch(c, "nn_relu_mask");
+      conv<true>(c, B, co, ci, H, W, dy, nullptr, nullptr, params + offs[k], nullptr,
+                 reinterpret_cast<float*>(acts[k - 1].p), dx, 0);
       std::swap(dyb, dxb);
       dy = reinterpret_cast<float*>(dyb.p);
     }

@@ -15,6 +15,7 @@ struct Net {
   int64_t nparam = 0;
   int64_t t = 0;                 // Adam steps taken
   float out_scale = 1.f;         // the network predicts y / out_scale
+  DBuf store;                    // device memory of the next two rows, from the context's pool
   float *params = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;   // device, nparam each
   float *shift = nullptr, *scale = nullptr;                               // device, c_in each
   std::vector<int> ci_, co_;     // channels per layer
