@@ -1158,6 +1158,7 @@ qtt_mps* zipup_hadamard(Ctx& c, const qtt_mps* a, const qtt_mps* b, int chi) {
 
 void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev) {
   QTT_CHECK_ARG(a->n == b->n && a->d == b->d, "dot: shape mismatch");
+  if (dot_fused(c, a, b, out_dev)) return;
   const int n = a->n, d = a->d;
   DBuf E(&c, 1);
   fill(c, E.p, 1, 1.0);
