@@ -187,8 +187,8 @@ int qtt_ctx_profile(qtt_ctx* ctx, int on, double* ms_out, double* flops_out, int
  * with momentum, unused, Poisson, projection -- row 5 = outside any phase; column k = kernel
  * class k), and launches_out[6] (kernel launches enqueued in each row).  Either may be NULL. */
 int qtt_ctx_profile_phases(qtt_ctx* ctx, double* ms_out, int64_t* launches_out);
-/* Limit (seconds, > 0) of every bounded device wait of this context: the grid barriers of the
- * cooperative CG solves (default 2 s).  A wait that runs out makes its kernel leave at once;
+/* Limit (seconds, > 0) of every bounded device wait of this context: the barriers of the one-kernel
+ * CG solves (default 2 s).  A wait that runs out makes its kernel leave at once;
  * the solve then ends with QTT_SOLVE_TIMEOUT and the call returns QTT_ERR_TIMEOUT, with the
  * context still usable.  Takes effect for work enqueued afterwards (a captured step keeps the
  * limit it was captured with: set it before the first fractional_step or after
@@ -199,8 +199,9 @@ int qtt_ctx_set_wait_limit(qtt_ctx* ctx, double seconds);
  * the bonds allow it (bonds <= 128, operator bonds <= 16, d <= 4).  Mode 3 does the same but,
  * on the context's own stream with left bond <= 64 and the tensor-core product mode
  * (qtt_ctx_set_gemm_mode 0), runs both contractions as exact digit-split products on the
- * tensor cores.  Mode 0 (default) takes mode 3 at sites whose bonds multiply to at least 4096
- * and mode 2 elsewhere.  Mode 1 launches one kernel per contraction and per CG update.  All give
+ * tensor cores.  Mode 0 (default) takes mode 3 at sites whose bonds multiply to at least 4096,
+ * one thread-block cluster (hardware barriers) where they multiply to at most 256 and mode 2
+ * elsewhere.  Mode 1 launches one kernel per contraction and per CG update.  All give
  * the same iterates up to rounding order.  Returns QTT_ERR_ARG for another mode. */
 int qtt_ctx_set_cg_mode(qtt_ctx* ctx, int mode);
 

@@ -108,6 +108,12 @@ void cg_tc_init_attributes();
 void cg_tc(Ctx& c, const double* L, const double* W, const double* R, const double* b, double* x, int r0, int r1,
            int w0, int w1, int d, int iters, const double* tol_dev, int* total_dev, const double* dinv);
 
+// The same solve of a small site in one cluster (qtt_cg_team.cu), the preconditioner formed inside: x from xin, the
+// solution to xout.
+bool cg_team_fits(int r0, int r1, int w0, int w1, int d);
+void cg_team(Ctx& c, const double* L, const double* W, const double* R, const double* b, const double* xin, double* xout,
+             int r0, int r1, int w0, int w1, int d, int iters, const double* tol_dev, int* total_dev);
+
 void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev);
 // The same in one launch (qtt_dot.cu); false if the bonds are beyond what it takes.
 bool dot_fused(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev);

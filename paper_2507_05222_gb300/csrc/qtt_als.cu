@@ -414,9 +414,14 @@ void als(Ctx& c, const qtt_mpo* A, const std::vector<Term>& rhs, qtt_mps* x, con
     // mode 3: tensor cores wherever the kernel fits
     const int mode = c.root->cg_mode;
     const bool tc = (mode == 3 || (mode == 0 && int64_t(r0) * r1 >= 4096)) && cg_tc_fits(c, r0, r1, w0, w1, d);
-    DBuf bvec(&c, nel), xk(&c, nel), dinv(&c, nel);
+    DBuf bvec(&c, nel), xk(&c, nel);
     for (size_t t = 0; t < rhs.size(); ++t)
       local_target(c, rhs[t], E.L[t][k].p, E.R[t][k + 1].p, r0, r1, k, rhs[t].coef, t == 0 ? 0.0 : 1.0, bvec.p);
+    if (mode == 0 && cg_team_fits(r0, r1, w0, w1, d)) {
+      cg_team(c, LA[k].p, A->core(k), RA[k + 1].p, bvec.p, x->core(k), xk.p, r0, r1, w0, w1, d, o.cg_max_iter, cg_tol, total);
+      return xk;
+    }
+    DBuf dinv(&c, nel);
     copy(c, xk.p, x->core(k), nel);
     k_local_dinv<<<grid_for(nel, 256), 256, 0, c.stream>>>(LA[k].p, A->core(k), RA[k + 1].p, r0, r1, w0, w1, d, dinv.p);
     after_launch(c, "local_dinv");

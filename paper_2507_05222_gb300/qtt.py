@@ -282,8 +282,8 @@ class Context:
 
     def set_cg_mode(self, mode: int):
         """ALS local CG solves: 0 (default) one cooperative kernel per solve, its contractions on
-        the tensor cores at full-bond sites (bonds multiplying to >= 4096) and on the FP64 pipe
-        elsewhere; 1 one kernel per stage; 2 the cooperative kernel on the FP64 pipe only; 3 the
+        the tensor cores at full-bond sites (bonds multiplying to >= 4096), one cluster at small
+        sites (<= 256) and the FP64 pipe elsewhere; 1 one kernel per stage; 2 the cooperative kernel on the FP64 pipe only; 3 the
         tensor-core contractions wherever the cooperative kernel fits."""
         _check(lib().qtt_ctx_set_cg_mode(self.h, int(mode)))
 
