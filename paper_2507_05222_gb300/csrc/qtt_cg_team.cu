@@ -5,11 +5,9 @@
 //     for the CTA's own b, written into every team member's shared memory (DSMEM); barrier;
 //   Ap[c, s, e] = sum_{v,b} T2[s, v, b] R[e, v, b] for the CTA's own e.
 // The CTA that computes Ap[c, s, e] owns x, r, p, Ap and the preconditioner of those elements in
-// its shared memory.  Each iteration has one reduction over the cluster (p.Ap, r.r, r.z and the products that
-// give the next r.r and r.z: rr' = rr - 2 a r.Ap + a^2 Ap.Ap, rz' likewise), so that alpha and beta
-// are known after one barrier; r.r and r.z themselves are formed anew every iteration, and a
-// predicted r.r is trusted to end the solve only where it did not cancel.  A second barrier
-// publishes p.
+// its shared memory.  The recurrences are those of qtt_cg.cu with two barriers an iteration: the first
+// carries the sums of p.Ap, the second those of r.r and r.z together with z, from which every CTA
+// forms the next p = z + beta p of the b that it needs in its own shared memory.
 //
 // What bounds it: barriers and FP64 latency (64 clocks an operation, 110 a shuffle-sum level).
 // qtt_cg.cu's kernels take three to four grid barriers of 1.3 us and five block reductions an
@@ -30,7 +28,7 @@ namespace qtt {
 namespace {
 
 constexpr int TM_THREADS = 256;
-constexpr int TM_SUMS = 7;        // p.Ap, r.r, r.z, r.Ap, Ap.Ap, r.D.Ap, Ap.D.Ap
+constexpr int TM_SUMS = 3;        // at most: b.b, r.r, r.z
 constexpr int TM_POISON = -(1 << 29);
 constexpr size_t TM_SMEM = 200 * 1024;
 constexpr int TM_CLUSTER = 16, TM_ELEMS = 256;
@@ -46,8 +44,8 @@ struct TeamArgs {
   const double* b;
   const double* xin;
   double* xout;
-  double* p;                      // published direction (r0, d, r1)
-  double* part;                   // 2 x TM_SUMS x gridDim.x
+  double* z;                      // published D r (r0, d, r1)
+  double* part;                   // 2 x TM_SUMS x gridDim.x: the sums of the two barriers
   unsigned long long limit_ns;
   int* total;
   double* flops;
@@ -75,26 +73,20 @@ __device__ __forceinline__ double tm_warp_sum(double v) {
   return v;
 }
 
-// Lanes that share an output: as many as the threads allow, at most K and a warp.
-__device__ __forceinline__ int tm_lanes(int outs, int K) {
+// Lanes that share an output of the last contraction: as many as the threads allow, at most the 16 of
+// qtt_cg.cu's stage B.
+__device__ __forceinline__ int tm_lanes(int outs) {
   int l = 1;
-  while (l < 32 && outs * l * 2 <= TM_THREADS && l * 2 <= K) l *= 2;
+  while (l < 16 && outs * l * 2 <= TM_THREADS) l *= 2;
   return l;
 }
 
-// sum_k x[k sx] y[k sy] over lanes l, l + nl, ... with two partial sums, then over the lanes.
+// sum_k x[k sx] y[k sy] over lanes l, l + nl, ..., then over the lanes.
 template <bool YG>
 __device__ __forceinline__ double tm_dot(const double* x, int sx, const double* y, int sy, int K, int l, int nl, bool in) {
-  double s0 = 0.0, s1 = 0.0;
-  if (in) {
-    int k = l;
-    for (; k + nl < K; k += 2 * nl) {
-      s0 = fma(x[k * sx], YG ? __ldg(y + k * sy) : y[k * sy], s0);
-      s1 = fma(x[(k + nl) * sx], YG ? __ldg(y + (k + nl) * sy) : y[(k + nl) * sy], s1);
-    }
-    if (k < K) s0 = fma(x[k * sx], YG ? __ldg(y + k * sy) : y[k * sy], s0);
-  }
-  double s = s0 + s1;
+  double s = 0.0;
+  if (in)
+    for (int k = l; k < K; k += nl) s = fma(x[k * sx], YG ? __ldg(y + k * sy) : y[k * sy], s);
   for (int o = nl >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
 }
@@ -103,31 +95,38 @@ struct TeamSmem {
   double *P, *L, *W, *T1, *T2, *R, *x, *r, *p, *Ap, *di;
 };
 
-// Ap of this CTA's elements from the vector V (r0, d, r1) in global memory.
-__device__ void tm_apply(const TeamArgs& a, const TeamSmem& s, const double* V, int team, int rank) {
+// P[a, t, b of this CTA] <- V[a, t, b] + beta P, V (r0, d, r1) in global memory, read through L2 (other
+// CTAs write z in this launch).  beta = 0 takes V alone.
+__device__ void tm_direction(const TeamArgs& a, const TeamSmem& s, const double* V, double beta, int rank) {
+  const int bw = a.bw, b0 = rank * bw, nbw = max(0, min(bw, a.r1 - b0));
+  for (int e = threadIdx.x; e < a.r0 * a.d * nbw; e += TM_THREADS) {
+    const int row = e / nbw, bb = e - row * nbw;
+    const double v = __ldcg(V + size_t(row) * a.r1 + b0 + bb);
+    double* p = s.P + row * bw + bb;
+    *p = beta == 0.0 ? v : fma(beta, *p, v);
+  }
+}
+
+// Ap of this CTA's elements from the P of its team.
+__device__ void tm_apply(const TeamArgs& a, const TeamSmem& s, int team, int rank) {
   const int r0 = a.r0, r1 = a.r1, w0 = a.w0, w1 = a.w1, d = a.d, bw = a.bw, tid = threadIdx.x;
   const int e0 = rank * a.ew, new_ = max(0, min(a.ew, r1 - e0));
   const int K = w1 * r1, Kp = K + 1;
   const int b0 = rank * bw, nbw = max(0, min(bw, r1 - b0));
   cgrp::cluster_group cl = cgrp::this_cluster();
-  // P[a, t, b]: rows of bw, read through L2 (other CTAs write p in this launch)
-  for (int e = tid; e < r0 * d * nbw; e += TM_THREADS) {
-    const int row = e / nbw, bb = e - row * nbw;
-    s.P[row * bw + bb] = __ldcg(V + size_t(row) * r1 + b0 + bb);
-  }
   for (int q = 0; q < a.rows; ++q) {   // several rows only where a team is one CTA
     const int c = team + q * a.teams;
     const bool live = c < r0;
     __syncthreads();
     if (live) {   // T1[w, t, b]
-      const int outs = w0 * d * nbw, nl = tm_lanes(outs, r0), l = tid % nl;
+      // One thread an output, in the order of qtt_cg.cu's stage A: terms that cancel there cancel here.
+      // Sums split over lanes cost as much time (a shuffle level is 110 clocks, an fma 64) and took steps from
+      // rest (chi = 8) five times further from the oracle.
+      const int outs = w0 * d * nbw;
       const double* Lc = s.L + size_t(q) * w0 * r0;
-      for (int o0 = 0; o0 < outs; o0 += TM_THREADS / nl) {
-        const int o = o0 + tid / nl;
-        const bool in = o < outs;
-        const int oo = in ? o : 0, bb = oo % nbw, wt = oo / nbw, t = wt % d, w = wt / d;
-        const double v = tm_dot<false>(Lc + w * r0, 1, s.P + t * bw + bb, d * bw, r0, l, nl, in);
-        if (in && l == 0) s.T1[wt * bw + bb] = v;
+      for (int o = tid; o < outs; o += TM_THREADS) {
+        const int bb = o % nbw, wt = o / nbw, t = wt % d, w = wt / d;
+        s.T1[wt * bw + bb] = tm_dot<false>(Lc + w * r0, 1, s.P + t * bw + bb, d * bw, r0, 0, 1, true);
       }
     }
     __syncthreads();
@@ -148,7 +147,7 @@ __device__ void tm_apply(const TeamArgs& a, const TeamSmem& s, const double* V, 
     if (a.cs > 1) cl.sync();
     else __syncthreads();
     if (live) {   // Ap[s, e]
-      const int outs = d * new_, nl = tm_lanes(outs, K), l = tid % nl;
+      const int outs = d * new_, nl = tm_lanes(outs), l = tid % nl;
       for (int o0 = 0; o0 < outs; o0 += TM_THREADS / nl) {
         const int o = o0 + tid / nl;
         const bool in = o < outs;
@@ -162,34 +161,22 @@ __device__ void tm_apply(const TeamArgs& a, const TeamSmem& s, const double* V, 
   __syncthreads();
 }
 
-// Sums over the CTA's elements, one warp a quantity, into part[k gridDim.x + block] (two such arrays
-// in turn: a slow CTA may still read one while the next sums are written).
-__device__ void tm_sums(const TeamArgs& a, const TeamSmem& s, double* part, int nloc, bool first, const double* bv) {
+// Sums of f(k, i) over the CTA's elements for k < ns, one warp a quantity, into part[k gridDim.x + block].
+template <class F>
+__device__ __forceinline__ void tm_sums(double* part, int ns, int nloc, F f) {
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (k < TM_SUMS) {
+  if (k < ns) {
     double v = 0.0;
-    for (int i = lane; i < nloc; i += 32) {
-      const double r = s.r[i], ap = s.Ap[i];
-      double x, y;
-      if (first) {          // r.r, r.z and b.b
-        x = k == 0 ? bv[i] : r;
-        y = k == 0 ? bv[i] : k == 1 ? r : s.di[i] * r;
-        if (k > 2) { x = 0.0; y = 0.0; }
-      } else {
-        x = k == 0 ? s.p[i] : (k == 1 || k == 2 || k == 3 || k == 5) ? r : ap;
-        y = k == 0 || k == 3 || k == 4 ? ap : k == 1 ? r : k == 2 ? s.di[i] * r : s.di[i] * ap;
-      }
-      v = fma(x, y, v);
-    }
+    for (int i = lane; i < nloc; i += 32) v += f(k, i);
     v = tm_warp_sum(v);
     if (lane == 0) part[k * gridDim.x + blockIdx.x] = v;
   }
 }
 
 // The grid's sums (the same in every CTA), one warp a quantity.
-__device__ void tm_totals(const double* part, double* tot) {
+__device__ void tm_totals(const double* part, int ns, double* tot) {
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31, G = gridDim.x;
-  if (k < TM_SUMS) {
+  if (k < ns) {
     double v = 0.0;
     for (int i = lane; i < G; i += 32) v += __ldcg(part + k * G + i);
     v = tm_warp_sum(v);
@@ -253,59 +240,62 @@ __global__ void __launch_bounds__(TM_THREADS) k_cg_team(const __grid_constant__ 
     s.p[i] = 0.0;
     s.Ap[i] = 0.0;
   }
+  // r = b - A x, p = z = D r
+  tm_direction(a, s, a.xin, 0.0, rank);
+  tm_apply(a, s, team, rank);
+  for (int i = tid; i < ncap; i += TM_THREADS) {
+    const int e = i % a.ew, s_ = (i / a.ew) % d, q = i / (a.ew * d), c = team + q * a.teams;
+    if (c < r0 && e < new_) {
+      const size_t g = (size_t(c) * d + s_) * r1 + e0 + e;
+      const double bv = __ldg(a.b + g), re = bv - s.Ap[i], z = s.di[i] * re;
+      s.r[i] = re;
+      s.p[i] = z;
+      s.Ap[i] = bv;          // for b.b
+      a.z[g] = z;
+    }
+  }
+  __syncthreads();
+  double* const part0 = a.part;
+  double* const part1 = a.part + TM_SUMS * gridDim.x;
+  tm_sums(part1, 3, ncap, [&](int k, int i) {
+    const double x = k == 0 ? s.Ap[i] : s.r[i];
+    return k == 2 ? x * (s.di[i] * x) : x * x;
+  });
+  tm_sync(a, &err);
+  tm_totals(part1, 3, tot);
+  const double tol2bb = __ldg(a.tol) * __ldg(a.tol) * tot[0];
+  double rr = tot[1], rz = tot[2], beta = 0.0;
   int count = 0;
-  {
-    // ---- r = b - A x, p = z
-    tm_apply(a, s, a.xin, team, rank);
+  for (int it = 0; it < a.iters && rr > tol2bb && rr > 0.0; ++it) {   // the same decisions in every CTA
+    tm_direction(a, s, a.z, beta, rank);
+    tm_apply(a, s, team, rank);
+    tm_sums(part0, 1, ncap, [&](int, int i) { return s.p[i] * s.Ap[i]; });
+    tm_sync(a, &err);
+    tm_totals(part0, 1, tot);
+    const double pap = tot[0];
+    if (!(pap > 0.0)) break;
+    const double alpha = rz / pap;
+    count += 1;
     for (int i = tid; i < ncap; i += TM_THREADS) {
       const int e = i % a.ew, s_ = (i / a.ew) % d, q = i / (a.ew * d), c = team + q * a.teams;
       if (c < r0 && e < new_) {
-        const size_t g = (size_t(c) * d + s_) * r1 + e0 + e;
-        const double bv = __ldg(a.b + g), re = bv - s.Ap[i], z = s.di[i] * re;
+        const double re = fma(-alpha, s.Ap[i], s.r[i]);
+        s.x[i] = fma(alpha, s.p[i], s.x[i]);
         s.r[i] = re;
-        s.p[i] = z;
-        s.Ap[i] = bv;          // for b.b below
-        a.p[g] = z;
+        a.z[(size_t(c) * d + s_) * r1 + e0 + e] = s.di[i] * re;
       }
     }
     __syncthreads();
-    tm_sums(a, s, a.part, ncap, true, s.Ap);
+    tm_sums(part1, 2, ncap, [&](int k, int i) {
+      const double x = s.r[i];
+      return k == 1 ? x * (s.di[i] * x) : x * x;
+    });
     tm_sync(a, &err);
-    tm_totals(a.part, tot);
-    const double bb = tot[0], tol2 = __ldg(a.tol) * __ldg(a.tol);
-    double rr = tot[1];
-    bool active = rr > tol2 * bb && rr > 0.0;
-    for (int it = 0; it < a.iters && active; ++it) {
-      tm_apply(a, s, a.p, team, rank);
-      double* part = a.part + ((it + 1) & 1) * TM_SUMS * gridDim.x;
-      tm_sums(a, s, part, ncap, false, nullptr);
-      tm_sync(a, &err);
-      tm_totals(part, tot);
-      const double pap = tot[0], rz = tot[2];
-      rr = tot[1];
-      if (it > 0 && !(rr > tol2 * bb && rr > 0.0)) break;   // the last step did it (its prediction had cancelled)
-      if (!(pap > 0.0)) break;                               // the same decision in every CTA
-      const double alpha = rz / pap;
-      const double rn = fma(alpha, fma(alpha, tot[4], -2.0 * tot[3]), rr);
-      const double rzn = fmax(fma(alpha, fma(alpha, tot[6], -2.0 * tot[5]), rz), 0.0);
-      const double beta = rzn / rz;
-      count += 1;
-      // a prediction below 1e-8 of r.r is mostly rounding: go on, the next sums decide
-      if (rn > 1e-8 * rr) active = rn > tol2 * bb;
-      for (int i = tid; i < ncap; i += TM_THREADS) {
-        const int e = i % a.ew, s_ = (i / a.ew) % d, q = i / (a.ew * d), c = team + q * a.teams;
-        if (c < r0 && e < new_) {
-          const double p = s.p[i], re = fma(-alpha, s.Ap[i], s.r[i]);
-          s.x[i] = fma(alpha, p, s.x[i]);
-          s.r[i] = re;
-          const double pn = fma(beta, p, s.di[i] * re);
-          s.p[i] = pn;
-          a.p[(size_t(c) * d + s_) * r1 + e0 + e] = pn;
-        }
-      }
-      if (!active) break;
-      tm_sync(a, &err);
-    }
+    tm_totals(part1, 2, tot);
+    rr = tot[0];
+    beta = tot[1] / rz;
+    rz = tot[1];
+    for (int i = tid; i < ncap; i += TM_THREADS) s.p[i] = fma(beta, s.p[i], s.di[i] * s.r[i]);
   }
   for (int i = tid; i < ncap; i += TM_THREADS) {
     const int e = i % a.ew, s_ = (i / a.ew) % d, q = i / (a.ew * d), c = team + q * a.teams;
@@ -368,8 +358,8 @@ int team_max_clusters(int cs, size_t smem) {
 }
 
 // One cluster up to r0 r1 = 256.  Poisson solves on 10 bits, against the cooperative kernel of qtt_cg.cu
-// (same iterations): all bonds <= 8 13.2 -> 9.6 ms (210 iterations, 4 sweeps), <= 12 11.6 -> 8.3 ms, <= 16
-// 10.4 -> 7.8 ms.  Larger sites want more than 16 CTAs and stay with the cooperative kernels.
+// (same iterations): all bonds <= 8 13.0 -> 9.5 ms (210 iterations, 4 sweeps), <= 12 11.4 -> 8.3 ms, <= 16
+// 10.3 -> 7.7 ms.  Larger sites want more than 16 CTAs and stay with the cooperative kernels.
 bool cg_team_plan(int r0, int r1, int w0, int w1, int d, TeamPlan& p) {
   if (!(r0 >= 1 && r1 >= 1 && r0 * int64_t(r1) <= TM_ELEMS && w0 >= 1 && w1 >= 1 && w0 <= 16 && w1 <= 16 && d >= 1 && d <= 4))
     return false;
@@ -400,13 +390,13 @@ void cg_team(Ctx& c, const double* L, const double* W, const double* R, const do
              int r0, int r1, int w0, int w1, int d, int iters, const double* tol_dev, int* total_dev) {
   TeamPlan p;
   QTT_CHECK_ARG(cg_team_plan(r0, r1, w0, w1, d, p), "cg_team: shape outside the supported range");
-  DBuf dir(&c, size_t(r0) * d * r1), part(&c, size_t(2 * TM_SUMS) * p.grid);
+  DBuf zbuf(&c, size_t(r0) * d * r1), part(&c, size_t(2 * TM_SUMS) * p.grid);
   TeamArgs a;
   a.r0 = r0; a.r1 = r1; a.w0 = w0; a.w1 = w1; a.d = d; a.iters = iters;
   a.cs = p.cs; a.teams = p.teams; a.bw = p.bw; a.ew = p.ew; a.rows = p.rows; a.rres = p.rres;
   a.tol = tol_dev;
   a.L = L; a.W = W; a.R = R; a.b = b; a.xin = xin; a.xout = xout;
-  a.p = dir.p; a.part = part.p;
+  a.z = zbuf.p; a.part = part.p;
   a.limit_ns = c.root->wait_ns;
   a.total = total_dev;
   a.flops = c.root->prof.on ? c.root->prof.dev_flops : nullptr;
