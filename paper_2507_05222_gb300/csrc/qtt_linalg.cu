@@ -147,63 +147,48 @@ __global__ void __launch_bounds__(256) k_qr(int m, int n, int trans, const doubl
 }
 
 // ------------------------------------------------------------------ cluster Householder QR (FP64)
-// Same factorisation and conventions as k_qr (beta = -sign(alpha) ||x||, unit-diagonal
-// reflectors, thin Q), for m >= n, organised as a blocked right-looking QR over a cluster of
-// cs CTAs.  CTA q owns columns [q nb, q nb + nb) and holds them in shared memory for the
-// whole factorisation; panel p is CTA p's column block.
-//   R phase, for p = 0 .. cs-1: CTA p factors its (already updated) panel with one warp and
-//     forms the compact-WY factor T_p (H_{j0} ... H_{j0+w-1} = I - V_p T_p V_p^T); after a
-//     cluster barrier every CTA q > p reads V_p and T_p from CTA p's shared memory (DSMEM)
-//     and updates its columns, A_q <- (I - V_p T_p^T V_p^T) A_q.
-//   Q phase: column block q of Q = H_0 ... H_{n-1} [I; 0] only sees panels p <= q, so each CTA
-//     accumulates its own columns of Q backwards from the final V_p, T_p with no further
-//     synchronisation; a last cluster barrier keeps every CTA's shared memory alive until the
-//     others have read it.
+// Same factorisation and conventions as k_qr (beta = -sign(alpha) ||x||, thin Q), for m >= n, over a
+// cluster of cs CTAs.  CTA q owns columns [q nb, q nb + nb) (panel q) in shared memory.
+//   R phase: CTA p forms its reflectors one after another.  Reflectors are left unnormalised,
+//     H = I - inv u u^T, u = x - beta e_r, inv = 1 / (||x|| (||x|| + |alpha|)), so x below the pivot
+//     is u and the products x . y with the panel's other columns come from the same reduction as
+//     x . x: one reduction a column.  As soon as a reflector is formed its owner arrives on a
+//     barrier of every later CTA, which reads it (DSMEM) and updates its columns, one warp each,
+//     while the owner forms the next one.
+//   Q phase: column block q of Q = H_0 ... H_{n-1} [I; 0] only sees panels p <= q (compact WY with
+//     T_p, formed by CTA p after its panel).  A CTA does it right after its own panel, beside the
+//     R phase of the later ones; the last cs / 4 panels, whose Q would be left over at the end, are
+//     split into four groups of columns, for their owner and three CTAs that are done by then.
+// Each barrier is used once and only later CTAs wait, on earlier ones, so the waits end; they are
+// bounded all the same (a wait that runs out gives NaN).
+// Columns are scaled by powers of two to a largest entry in [1, 2) (R's columns scaled back: exact),
+// so that the squares and products above neither overflow nor underflow.
+// What bounds it: the serial chain of FP64 instructions.  Each takes its sub-partition 64 clocks, dependent or
+// not and whatever its active lanes, so the kernel is written for few of them on the longest chain.  A
+// column of a panel takes ~2.9k clocks: the dot product 1.1k, the scalars 1.2k, the update 0.6k.
+// A blocked right-looking form with normalised reflectors (two reductions a column, a block update
+// and a Q phase behind cluster barriers) took, against this one, in us: 128 x 64 275 -> 141, 64 x 64 217 -> 136,
+// 64 x 32 115 -> 70, 32 x 16 52 -> 37, 256 x 128 839 -> 453, 128 x 128 545 -> 318, 200 x 20 105 -> 58.
 // Shared layout (doubles): Acol | Qcol | Vb (m x nb each, column-major) | T | Tb | W | W2
-// (nb x nb each) | tau (nb).
+// (nb x nb each) | ud (nb).
 constexpr int QRC_THREADS = 256;
 
-// 1/sqrt(q) and 1/x by Newton-Raphson from the hardware's approximate FP64 reciprocal (square
-// root), two quadratically convergent steps each (~20 correct bits -> beyond 53).  An FP64
-// division or square root is a sequence of ~10 dependent FP64 operations, ~650 cycles on this
-// part; these take 3 x 64 (reciprocal) and 6 x 64 (reciprocal square root) cycles.  Results are
-// within a few ulp of the correctly rounded ones (checked against CUDA's by qtt_check_recip).
+// 1/x and 1/sqrt(x) from the hardware's approximate FP64 reciprocal (square root), ~20 correct bits,
+// by one third-order step each: with e = 1 - x y (or 1 - x y^2), y (1 + e + e^2) and
+// y (1 + e / 2 + 3 e^2 / 8) are good to e^3.  An FP64 division or square root is a sequence of ~10
+// dependent FP64 operations, ~650 cycles on this part; these take 3 x 64 and 4 x 64 cycles.  Results
+// are within a few ulp of the correctly rounded ones (checked against CUDA's by qtt_check_recip).
 __device__ __forceinline__ double rcp_nr(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ double rsqrt_nr(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double r = fma(-x * y, y, 1.0);
-  y = fma(0.5 * y, r, y);
-  r = fma(-x * y, y, 1.0);
-  return fma(0.5 * y, r, y);
-}
-
-// Householder scalars of a column with pivot alpha and sum of squares sigma below it (LAPACK
-// convention): beta = -sign(alpha) ||x||, t = (beta - alpha) / beta = 1 + |alpha| / ||x||,
-// scale = 1 / (alpha - beta) = sign(alpha) / (|alpha| + ||x||).  sigma = 0: identity reflector.
-__device__ __forceinline__ void householder_scalars(double alpha, double sigma, double& beta, double& t,
-                                                    double& scale) {
-  if (sigma == 0.0) {
-    t = 0.0;
-    beta = alpha;
-    scale = 0.0;
-    return;
-  }
-  const double q = fma(alpha, alpha, sigma);
-  const double g = rsqrt_nr(q);
-  const double nrm = q * g;
-  const double aa = fabs(alpha);
-  beta = alpha >= 0.0 ? -nrm : nrm;
-  t = fma(aa, g, 1.0);
-  const double rd = rcp_nr(aa + nrm);
-  scale = alpha >= 0.0 ? rd : -rd;
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 __global__ void k_check_recip(int n, const double* __restrict__ x, double* __restrict__ err) {
@@ -239,11 +224,12 @@ __global__ void k_check_recip(int n, const double* __restrict__ x, double* __res
 __host__ __device__ constexpr size_t qrc_smem_doubles(int m, int nb) {
   return size_t(3) * m * nb + 4 * size_t(nb) * nb + nb;
 }
+constexpr int QRC_MAX_CLUSTER = 16, QRC_MAX_NB = 16;
 
-// X(i, c) (i >= j0, c < ncols, column-major with leading dimension m) <- (I - V op(T) V^T) X,
-// op(T) = T^T when transT, else T.  V: m x wp (rows >= j0 valid), T: wp x wp upper triangular
-// with leading dimension nb.  Called by every thread of the CTA; ends with a CTA barrier.
-__device__ void qrc_apply_block(int m, int nb, int j0, int wp, int ncols, const double* V, const double* T, bool transT,
+// X(i, c) (i >= j0, c < ncols, column-major with leading dimension m) <- (I - V T V^T) X.
+// V: m x wp (rows >= j0 valid), T: wp x wp upper triangular with leading dimension
+// nb.  Called by every thread of the CTA; ends with a CTA barrier.
+__device__ void qrc_apply_block(int m, int nb, int j0, int wp, int ncols, const double* V, const double* T,
                                 double* X, double* W, double* W2) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nd = wp * ncols;
@@ -265,11 +251,7 @@ __device__ void qrc_apply_block(int m, int nb, int j0, int wp, int ncols, const 
   if (tid < nd) {
     const int l = tid / ncols, c = tid % ncols;
     double s = 0.0;
-    if (transT) {
-      for (int l2 = 0; l2 <= l; ++l2) s += T[l2 * nb + l] * W[l2 * ncols + c];
-    } else {
-      for (int l2 = l; l2 < wp; ++l2) s += T[l * nb + l2] * W[l2 * ncols + c];
-    }
+    for (int l2 = l; l2 < wp; ++l2) s += T[l * nb + l2] * W[l2 * ncols + c];
     W2[tid] = s;
   }
   __syncthreads();
@@ -283,19 +265,210 @@ __device__ void qrc_apply_block(int m, int nb, int j0, int wp, int ncols, const 
   __syncthreads();
 }
 
-// Copy panel p's reflectors (unit diagonal, zeros above, from the factored columns src) and
-// its T into the local buffers Vb, Tb.  Ends with a CTA barrier.
-__device__ void qrc_fetch_panel(int m, int nb, int j0, int wp, const double* src, const double* srcT, double* Vb,
-                                double* Tb) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int mr = m - j0;
-  for (int e = tid; e < mr * wp; e += nt) {
-    const int l = e / mr, i = j0 + e % mr;
-    const int diag = j0 + l;
-    Vb[size_t(l) * m + i] = (i < diag) ? 0.0 : (i == diag ? 1.0 : src[size_t(l) * m + i]);
+__device__ __forceinline__ uint32_t qrc_smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+// Arrive on the barrier at the same place in CTA `rank` of the cluster; what this CTA wrote before its
+// last CTA barrier is visible to whoever sees the arrival.
+__device__ __forceinline__ void qrc_signal(const uint64_t* bar, int rank) {
+  asm volatile(
+      "{\n\t.reg .b32 remote;\n\t"
+      "mapa.shared::cluster.u32 remote, %0, %1;\n\t"
+      "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(qrc_smem_addr(bar)), "r"(rank)
+      : "memory");
+}
+// Wait for the one arrival on an own barrier; false after some 4 million tries.
+__device__ __forceinline__ bool qrc_wait(const uint64_t* bar) {
+  for (int k = 0; k < (1 << 22); ++k) {
+    int done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+        "selp.s32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(qrc_smem_addr(bar))
+        : "memory");
+    if (done) return true;
   }
-  for (int e = tid; e < wp * nb; e += nt) Tb[e] = srcT[e];
-  __syncthreads();
+  return false;
+}
+
+// 2^-e of a column whose largest entry lies in [2^e, 2^(e+1)) from the largest high word without its
+// sign; 1 for a zero column and one that is not finite.
+__device__ __forceinline__ double qrc_scale(unsigned int hi, double& back) {
+  int b = int(hi >> 20);
+  if (hi == 0u || b == 2047) {
+    back = 1.0;
+    return 1.0;
+  }
+  b = min(max(b, 1), 2045);
+  back = __hiloint2double(b << 20, 0);             // 2^(b - 1023)
+  return __hiloint2double((2046 - b) << 20, 0);    // 2^(1023 - b)
+}
+
+// Rows r + lane + 32 t (t < 4) of a column; a chunk of 32 rows that lies beyond m is skipped by the whole
+// warp in what follows: an FP64 instruction takes its 64 clocks for idle lanes as well.
+__device__ __forceinline__ void qrc_load4(const double* u, int r, int m, int lane, double (&a)[4]) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) a[t] = r + lane + 32 * t < m ? u[r + lane + 32 * t] : 0.0;
+}
+// sum_{i > r} u_i y_i of a column by one warp
+__device__ __forceinline__ double qrc_dot(const double* u, const double* y, int r, int m, int lane) {
+  double d = 0.0;
+  for (int r0 = r; r0 < m; r0 += 128) {
+    double a[4], b[4];
+    qrc_load4(u, r0, m, lane, a);
+    qrc_load4(y, r0, m, lane, b);
+    if (r0 == r && lane == 0) a[0] = b[0] = 0.0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (r0 + 32 * t < m) d = fma(a[t], b[t], d);
+  }
+  return warp_sum(d);
+}
+// y_i -= wk u_i for i >= r, u_r = us
+__device__ __forceinline__ void qrc_update(const double* u, double us, double* y, int r, int m, int lane, double wk) {
+  for (int r0 = r; r0 < m; r0 += 128) {
+    double a[4], b[4];
+    qrc_load4(u, r0, m, lane, a);
+    qrc_load4(y, r0, m, lane, b);
+    if (r0 == r && lane == 0) a[0] = us;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (r0 + 32 * t < m) {
+        b[t] = fma(-wk, a[t], b[t]);
+        if (r0 + lane + 32 * t < m) y[r0 + lane + 32 * t] = b[t];
+      }
+  }
+}
+
+// Column cc of Q = H_0 ... H_{n-1} [I; 0] by WPC warps in registers (rows lane + 32 (sub + WPC t), t < RPL,
+// m <= 32 WPC RPL): blocks of four reflectors, panels P, P - 1, ..., 0, each block's V read from its
+// owner (DSMEM) while the block before is applied (RPL <= 4).  The 4 x 4 diagonal blocks of T_p are the T
+// of such blocks; lane l (mod 4) keeps row l.
+template <int RPL>
+struct QrcBlock {
+  double v[4][RPL], t[4];
+};
+template <int RPL, int WPC>
+__device__ __forceinline__ void qrc_load_block(QrcBlock<RPL>& b, const double* A, const double* T, const double* ud, int m,
+                                               int nb, int j0, int l0, int wp, int lane, int sub) {
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const int diag = j0 + l0 + l;
+    const bool in = l0 + l < wp;
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) {
+      const int i = lane + 32 * (sub + WPC * t);
+      double x = 0.0;
+      if (in && i > diag && i < m) x = A[size_t(l0 + l) * m + i];
+      if (in && i == diag) x = ud[l0 + l];
+      b.v[l][t] = x;
+    }
+  }
+  const int l = lane & 3;
+#pragma unroll
+  for (int l2 = 0; l2 < 4; ++l2) b.t[l2] = l <= l2 && l0 + l2 < wp ? T[(l0 + l) * nb + l0 + l2] : 0.0;
+}
+// red: this column's 2 x 4 x 4 doubles, blk counts its blocks (buffers in turn)
+template <int RPL, int WPC>
+__device__ __forceinline__ void qrc_apply4(const QrcBlock<RPL>& b, double (&x)[RPL], int lane, int sub, double* red, int group,
+                                           int blk) {
+  double d[4];
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    d[l] = b.v[l][0] * x[0];
+#pragma unroll
+    for (int t = 1; t < RPL; ++t) d[l] = fma(b.v[l][t], x[t], d[l]);
+  }
+  // four sums in six additions: lanes split over the values first; lane 8 l ends with sum l
+  const bool hi = lane & 16, h8 = lane & 8;
+  const double e0 = (hi ? d[2] : d[0]) + __shfl_xor_sync(0xffffffffu, hi ? d[0] : d[2], 16);
+  const double e1 = (hi ? d[3] : d[1]) + __shfl_xor_sync(0xffffffffu, hi ? d[1] : d[3], 16);
+  double f = (h8 ? e1 : e0) + __shfl_xor_sync(0xffffffffu, h8 ? e0 : e1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+  double w[4];
+  if (WPC > 1) {
+    double* buf = red + 16 * (blk & 1);
+    if ((lane & 7) == 0) buf[4 * (lane >> 3) + sub] = f;
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");
+    const double* my = buf + 4 * (lane & 3);
+    f = (my[0] + my[1]) + (my[2] + my[3]);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) w[l] = __shfl_sync(0xffffffffu, f, l);
+  } else {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) w[l] = __shfl_sync(0xffffffffu, f, 8 * l);
+  }
+  double z = b.t[0] * w[0];
+#pragma unroll
+  for (int l2 = 1; l2 < 4; ++l2) z = fma(b.t[l2], w[l2], z);
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const double zl = __shfl_sync(0xffffffffu, z, l);
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) x[t] = fma(-zl, b.v[l][t], x[t]);
+  }
+}
+template <int RPL, int WPC>
+__device__ void qrc_q_job(int m, int n, int nb, int trans, int q, int P, int cc0, int gw, const double* Acol, const double* T,
+                          const double* ud, const uint64_t* bar_t, bool bad, double* redall, double* Q) {
+  cgrp::cluster_group cl = cgrp::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / WPC, sub = warp % WPC;
+  double* red = redall + 32 * (WPC > 1 ? group : 0);
+  for (int c = group; c < gw; c += int(blockDim.x >> 5) / WPC) {
+    bool ok = true;
+    double x[RPL];
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) x[t] = lane + 32 * (sub + WPC * t) == cc0 + c ? 1.0 : 0.0;
+    auto load = [&](QrcBlock<RPL>& b, int p, int l0) {
+      if (p != q) ok = qrc_wait(bar_t + p) && ok;
+      qrc_load_block<RPL, WPC>(b, cl.map_shared_rank(Acol, p), cl.map_shared_rank(T, p), cl.map_shared_rank(ud, p), m, nb,
+                               p * nb, l0, min(nb, n - p * nb), lane, sub);
+    };
+    int p = P, l0 = ((min(nb, n - P * nb) - 1) / 4) * 4, blk = 0;
+    auto next = [&]() {          // all panels but the last have nb columns
+      l0 -= 4;
+      if (l0 < 0) {
+        --p;
+        l0 = ((nb - 1) / 4) * 4;
+      }
+    };
+    if (RPL <= 4) {
+      QrcBlock<RPL> b0, b1;
+      load(b0, p, l0);
+      next();
+      while (true) {
+        if (p >= 0) load(b1, p, l0);
+        qrc_apply4<RPL, WPC>(b0, x, lane, sub, red, group, blk++);
+        if (p < 0) break;
+        next();
+        if (p >= 0) load(b0, p, l0);
+        qrc_apply4<RPL, WPC>(b1, x, lane, sub, red, group, blk++);
+        if (p < 0) break;
+        next();
+      }
+    } else {
+      while (p >= 0) {
+        QrcBlock<RPL> b;
+        load(b, p, l0);
+        qrc_apply4<RPL, WPC>(b, x, lane, sub, red, group, blk++);
+        next();
+      }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) {
+      const int i = lane + 32 * (sub + WPC * t);
+      const double v = ok && !bad ? x[t] : __longlong_as_double(0x7ff8000000000000ll);
+      if (i < m) {
+        if (trans) Q[int64_t(cc0 + c) * m + i] = v;   // Q^T row-major (n x m)
+        else Q[int64_t(i) * n + cc0 + c] = v;         // Q row-major (m x n)
+      }
+    }
+  }
 }
 
 __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb, int trans, const double* __restrict__ Ain,
@@ -313,13 +486,24 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
   double* Tb = T + nb * nb;
   double* W = Tb + nb * nb;
   double* W2 = W + nb * nb;
-  double* tau = W2 + nb * nb;
+  double* ud = W2 + nb * nb;
+  __shared__ uint64_t bar_col[QRC_MAX_CLUSTER * QRC_MAX_NB];   // reflector s of an earlier panel formed
+  __shared__ uint64_t bar_t[QRC_MAX_CLUSTER];                  // T of another panel formed
+  __shared__ double s_red[64];   // qrc_apply4: two columns
+  __shared__ double s_sigma, s_back[QRC_MAX_NB], s_beta[QRC_MAX_NB], inv[QRC_MAX_NB];
+  __shared__ int s_bad;
   const double* A = Ain + mat * in_stride;
   double* Q = Qall + mat * q_stride;
   double* R = Rall ? Rall + mat * r_stride : nullptr;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps_all = nt >> 5;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
   const int c0 = q * nb;
   const int w = max(0, min(nb, n - c0));
+  for (int e = tid; e < n + cs; e += nt) {
+    const uint64_t* b = e < n ? bar_col + e : bar_t + (e - n);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(qrc_smem_addr(b)) : "memory");
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (tid == 0) s_bad = 0;
   for (int e = tid; e < m * w; e += nt) {
     if (trans) {
       const int c = e / m, i = e % m;
@@ -331,117 +515,196 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
   }
   for (int e = tid; e < nb * nb; e += nt) T[e] = 0.0;
   __syncthreads();
+  for (int c = warp; c < w; c += nwarps) {
+    double* x = Acol + size_t(c) * m;
+    unsigned int hi = 0;
+    for (int i = lane; i < m; i += 32) hi = max(hi, static_cast<unsigned int>(__double2hiint(x[i])) & 0x7fffffffu);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    double back;
+    const double f = qrc_scale(hi, back);
+    for (int i = lane; i < m; i += 32) x[i] *= f;
+    if (lane == 0) s_back[c] = back;
+  }
+  cl.sync();   // every CTA has started and its barriers are there
 
-  // ---- R phase
-  for (int p = 0; p < cs; ++p) {
-    const int j0 = p * nb;
-    const int wp = max(0, min(nb, n - j0));
-    if (p == q) {
-      // Panel factorisation.  Warp 0 forms reflector j; the other panel columns are then updated
-      // by one warp each (every warp sits on its own SM sub-partition and FP64 unit: one warp
-      // issues at most one FP64 instruction per ~64 cycles on this part).
-      for (int j = 0; j < w; ++j) {
-        const int r = j0 + j;
-        if (warp == 0) {
-          double* x = Acol + size_t(j) * m;
-          double part0 = 0.0, part1 = 0.0;
-          int i = r + 1 + lane;
-          for (; i + 32 < m; i += 64) {
-            part0 = fma(x[i], x[i], part0);
-            part1 = fma(x[i + 32], x[i + 32], part1);
-          }
-          if (i < m) part0 = fma(x[i], x[i], part0);
-          const double sigma = warp_sum(part0 + part1);
-          const double alpha = x[r];
-          double beta, t, scale;
-          householder_scalars(alpha, sigma, beta, t, scale);
-          __syncwarp();
-          for (int i2 = r + 1 + lane; i2 < m; i2 += 32) x[i2] *= scale;
-          if (lane == 0) {
-            x[r] = beta;
-            tau[j] = t;
-          }
-        }
-        __syncthreads();
-        for (int jj = j + 1 + warp; jj < w; jj += nwarps_all) {
-          const double* x = Acol + size_t(j) * m;
-          double* y = Acol + size_t(jj) * m;
-          double sdot = 0.0;
-          for (int i = r + 1 + lane; i < m; i += 32) sdot = fma(x[i], y[i], sdot);
-          sdot = (warp_sum(sdot) + y[r]) * tau[j];
-          __syncwarp();
-          if (lane == 0) y[r] -= sdot;
-          for (int i = r + 1 + lane; i < m; i += 32) y[i] -= sdot * x[i];
-        }
-        __syncthreads();
-      }
-      // T: T_ii = tau_i, T_{0:i, i} = -tau_i T_{0:i, 0:i} z_{0:i, i} with z_{l,i} = v_l . v_i,
-      // the w (w - 1) / 2 products one warp each, then the triangular recurrence in warp 0
-      const int npair = w * (w - 1) / 2;
-      for (int pidx = warp; pidx < npair; pidx += nwarps_all) {
-        int i = 1, base = 0;
-        while (base + i <= pidx) {
-          base += i;
-          ++i;
-        }
-        const int l = pidx - base;
-        const double* vi = Acol + size_t(i) * m;
-        const double* vl = Acol + size_t(l) * m;
-        double sdot = 0.0;
-        for (int row = j0 + i + 1 + lane; row < m; row += 32) sdot = fma(vl[row], vi[row], sdot);
-        sdot = warp_sum(sdot) + vl[j0 + i];
-        if (lane == 0) W[l * nb + i] = sdot;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        for (int i = 0; i < w; ++i) {
-          if (lane < i) {
-            double sacc = 0.0;
-            for (int l2 = lane; l2 < i; ++l2) sacc = fma(T[lane * nb + l2], W[l2 * nb + i], sacc);
-            T[lane * nb + i] = -tau[i] * sacc;
-          }
-          if (lane == 0) T[i * nb + i] = tau[i];
-          __syncwarp();
-        }
-      }
-    }
-    cl.sync();
-    if (q > p) {
-      qrc_fetch_panel(m, nb, j0, wp, cl.map_shared_rank(Acol, p), cl.map_shared_rank(T, p), Vb, Tb);
-      qrc_apply_block(m, nb, j0, wp, w, Vb, Tb, true, Acol, W, W2);
+  // ---- R phase: the reflectors of the earlier panels as they are formed, one warp a column
+  bool ok = true;
+  for (int s = 0; s < c0 && s < n && w > 0; ++s) {
+    const int p = s / nb, l = s - p * nb;
+    ok = qrc_wait(bar_col + s) && ok;
+    double* u = Vb + size_t(s & 1) * m;
+    const double* src = cl.map_shared_rank(Acol, p) + size_t(l) * m;
+    for (int i = s + 1 + tid; i < m; i += nt) u[i] = src[i];
+    const double us = cl.map_shared_rank(ud, p)[l], iv = cl.map_shared_rank(inv, p)[l];
+    __syncthreads();
+    for (int c = warp; c < w; c += nwarps) {
+      double* y = Acol + size_t(c) * m;
+      const double ys = y[s];
+      const double wk = fma(us, ys, qrc_dot(u, y, s, m, lane)) * iv;
+      __syncwarp();
+      qrc_update(u, us, y, s, m, lane, wk);
     }
   }
+  if (!ok) s_bad = 1;
+  __syncthreads();
+  if (s_bad)
+    for (int e = tid; e < m * w; e += nt) Acol[e] = __longlong_as_double(0x7ff8000000000000ll);
+  __syncthreads();
+  // ---- own panel: x_j . x_k for all k >= j at once, warp k % nwarps has column k
+  for (int j = 0; j < w; ++j) {
+    const int r = c0 + j;
+    const double* x = Acol + size_t(j) * m;
+    double dots[2];   // columns k = warp, warp + nwarps
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = warp + h * nwarps;
+      dots[h] = 0.0;
+      if (k >= j && k < w) {
+        const double* y = Acol + size_t(k) * m;
+        dots[h] = qrc_dot(x, y, r, m, lane);
+        if (k == j && lane == 0) s_sigma = dots[h];
+      }
+    }
+    __syncthreads();
+    const bool works = (warp >= j && warp < w) || (warp + nwarps >= j && warp + nwarps < w);
+    if (works) {
+      // LAPACK's convention: beta = -sign(alpha) ||x||.  Below 2^-960 (of a column scaled to 1) the
+      // reflector is the identity.  ||x|| comes straight from rsqrt_nr's correction of q y, and signs and
+      // limits are tested on the high words: an FP64 comparison costs as much as an fma.
+      const double alpha = x[r], sigma = s_sigma, aa = fabs(alpha);
+      const double qq = fma(alpha, alpha, sigma);
+      double y0;
+      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(qq));
+      const double n0 = qq * y0, e = fma(-n0, y0, 1.0);
+      const double nrm = fma(n0 * e, fma(0.375, e, 0.5), n0), tt = aa + nrm;
+      const bool idn = (static_cast<unsigned int>(__double2hiint(sigma)) & 0x7fffffffu) < 0x03f00000u;
+      const int ahi = __double2hiint(alpha);
+      const bool neg = ahi < 0 && ((ahi & 0x7fffffff) | __double2loint(alpha)) != 0;   // alpha < 0
+      const double iv = idn ? 0.0 : rcp_nr(nrm * tt);
+      const double beta = idn ? alpha : neg ? nrm : -nrm;
+      const double us = idn ? 0.0 : neg ? -tt : tt;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = warp + h * nwarps;
+        if (k > j && k < w) {
+          double* y = Acol + size_t(k) * m;
+          const double wk = idn ? 0.0 : fma(us, y[r], dots[h]) * iv;
+          __syncwarp();
+          qrc_update(x, us, y, r, m, lane, wk);
+        }
+      }
+      if (warp == j % nwarps && lane == 0) {
+        ud[j] = us;
+        inv[j] = iv;
+        s_beta[j] = beta;   // x[r] itself is still read by the other warps
+      }
+    }
+    __syncthreads();
+    const int to = tid - (nt - 32);   // by the last warp, which has no column of a 4-column panel
+    if (to > q && to < cs) qrc_signal(bar_col + r, to);
+  }
+  __syncthreads();
+  // T: T_ii = inv_i, T_{0:i, i} = -inv_i T_{0:i, 0:i} z_{0:i, i} with z_{l,i} = u_l . u_i, the
+  // w (w - 1) / 2 products one warp each, then the triangular recurrence in warp 0
+  const int npair = w * (w - 1) / 2;
+  for (int pidx = warp; pidx < npair; pidx += nwarps) {
+    int i = 1, base = 0;
+    while (base + i <= pidx) {
+      base += i;
+      ++i;
+    }
+    const int l = pidx - base;
+    const double* ui = Acol + size_t(i) * m;
+    const double* ul = Acol + size_t(l) * m;
+    double sdot = 0.0;
+    for (int row = c0 + i + 1 + lane; row < m; row += 32) sdot = fma(ul[row], ui[row], sdot);
+    sdot = fma(ul[c0 + i], ud[i], warp_sum(sdot));
+    if (lane == 0) W[l * nb + i] = sdot;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    for (int i = 0; i < w; ++i) {
+      if (lane < i) {
+        double sacc = 0.0;
+        for (int l2 = lane; l2 < i; ++l2) sacc = fma(T[lane * nb + l2], W[l2 * nb + i], sacc);
+        T[lane * nb + i] = -inv[i] * sacc;
+      }
+      if (lane == 0) T[i * nb + i] = inv[i];
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  if (tid != q && tid < cs) qrc_signal(bar_t + q, tid);
   if (R) {
     for (int e = tid; e < n * w; e += nt) {
       const int r = e / w, c = e % w;
-      R[int64_t(r) * n + c0 + c] = (r <= c0 + c) ? Acol[size_t(c) * m + r] : 0.0;
+      R[int64_t(r) * n + c0 + c] = r < c0 + c ? Acol[size_t(c) * m + r] * s_back[c] : r == c0 + c ? s_beta[c] * s_back[c] : 0.0;
     }
   }
 
-  // ---- Q phase: own columns of H_0 ... H_{n-1} [I; 0], panels q, q-1, ..., 0
-  for (int e = tid; e < m * w; e += nt) {
-    const int c = e / m, i = e % m;
-    Qcol[size_t(c) * m + i] = (i == c0 + c) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int p = q; p >= 0; --p) {
-    const int j0 = p * nb;
-    const int wp = max(0, min(nb, n - j0));
-    const double* srcA = (p == q) ? Acol : cl.map_shared_rank(Acol, p);
-    const double* srcT = (p == q) ? T : cl.map_shared_rank(T, p);
-    qrc_fetch_panel(m, nb, j0, wp, srcA, srcT, Vb, Tb);
-    qrc_apply_block(m, nb, j0, wp, w, Vb, Tb, false, Qcol, W, W2);
-  }
-  for (int e = tid; e < m * w; e += nt) {
-    if (trans) {
-      const int c = e / m, i = e % m;
-      Q[int64_t(c0 + c) * m + i] = Qcol[size_t(c) * m + i];   // Q^T row-major (n x m)
+  // ---- Q phase: (panel, column group) jobs of H_0 ... H_{n-1} [I; 0], panels P, P - 1, ..., 0
+  const int nsplit = cs / 4;
+  for (int job = 0; job < 2; ++job) {
+    int P = q, g0 = 0, gw = w;
+    if (job == 0) {
+      if (q >= cs - nsplit) {            // the owner's quarter of a split panel
+        const int gq = (w + 3) / 4;
+        g0 = min(w, 3 * gq);
+        gw = w - g0;
+      }
     } else {
-      const int i = e / w, c = e % w;
-      Q[int64_t(i) * n + c0 + c] = Qcol[size_t(c) * m + i];   // Q row-major (m x n)
+      if (q >= 3 * nsplit) break;        // helpers: CTA q has quarter q % 3 of panel cs - 1 - q / 3
+      P = cs - 1 - q / 3;
+      const int wP = max(0, min(nb, n - P * nb)), gq = (wP + 3) / 4;
+      g0 = min(wP, (q % 3) * gq);
+      gw = min(wP, g0 + gq) - g0;
     }
+    if (gw <= 0) continue;
+    const int cc0 = P * nb + g0;
+    // one or two columns: four warps each, so that the serial chain of panels is short
+#define QRC_JOB(rpl, wpc) qrc_q_job<rpl, wpc>(m, n, nb, trans, q, P, cc0, gw, Acol, T, ud, bar_t, s_bad != 0, s_red, Q)
+    if (m <= 256) {
+      if (gw <= 2) {
+        if (m <= 128) QRC_JOB(1, 4);
+        else QRC_JOB(2, 4);
+      } else {
+        if (m <= 128) QRC_JOB(4, 1);
+        else QRC_JOB(8, 1);
+      }
+      __syncthreads();
+      continue;
+    }
+#undef QRC_JOB
+    for (int e = tid; e < m * gw; e += nt) {
+      const int c = e / m, i = e % m;
+      Qcol[e] = (i == cc0 + c) ? 1.0 : 0.0;
+    }
+    for (int p = P; p >= 0; --p) {
+      const int j0 = p * nb, wp = max(0, min(nb, n - j0)), mr = m - j0;
+      if (p != q) ok = qrc_wait(bar_t + p) && ok;
+      const double* src = cl.map_shared_rank(Acol, p);
+      const double* srcT = cl.map_shared_rank(T, p);
+      const double* srcu = cl.map_shared_rank(ud, p);
+      for (int e = tid; e < mr * wp; e += nt) {
+        const int l = e / mr, i = j0 + e % mr, diag = j0 + l;
+        Vb[size_t(l) * m + i] = (i < diag) ? 0.0 : (i == diag ? srcu[l] : src[size_t(l) * m + i]);
+      }
+      for (int e = tid; e < wp * nb; e += nt) Tb[e] = srcT[e];
+      __syncthreads();
+      qrc_apply_block(m, nb, j0, wp, gw, Vb, Tb, Qcol, W, W2);
+    }
+    if (!ok) s_bad = 1;
+    __syncthreads();
+    const bool bad = s_bad != 0;
+    for (int e = tid; e < m * gw; e += nt) {
+      const int c = trans ? e / m : e % gw, i = trans ? e % m : e / gw;
+      const double v = bad ? __longlong_as_double(0x7ff8000000000000ll) : Qcol[size_t(c) * m + i];
+      if (trans) Q[int64_t(cc0 + c) * m + i] = v;   // Q^T row-major (n x m)
+      else Q[int64_t(i) * n + cc0 + c] = v;         // Q row-major (m x n)
+    }
+    __syncthreads();
   }
-  cl.sync();
+  cl.sync();   // no CTA leaves while another may read its panel
 }
 
 // ------------------------------------------------------------------ one-sided Jacobi SVD (FP64)
