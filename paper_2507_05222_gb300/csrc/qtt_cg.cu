@@ -22,8 +22,7 @@
 // Barrier: an arrival counter in device memory (reset before the launch); a waiting block polls
 // it for at most the context's wait limit (2 s unless set otherwise; global timer).  The
 // cooperative launch makes every block resident, so the bound is only a safety net: on expiry
-// the block sets the error flag,
-// every block leaves at its next barrier, and the iteration count is overwritten with a
+// the block sets the counter's top bit, every block leaves at its next barrier, and the iteration count is overwritten with a
 // negative value that the host turns into an error.  Data written by other blocks inside the
 // kernel are read with ld.global.cg (L2).
 #include <algorithm>
@@ -41,8 +40,7 @@ constexpr int CGP_MAX_W = 16;
 constexpr int CGP_MAX_D = 4;
 
 struct CgBar {
-  unsigned int count;   // arrivals so far (monotonic within a launch)
-  int error;            // set by a block that gave up waiting
+  unsigned long long count;      // arrivals so far (monotonic within a launch); top bit: a block gave up waiting
   unsigned long long limit_ns;   // how long a block waits at one barrier (the context's wait limit)
 };
 
@@ -67,25 +65,22 @@ struct CgArgs {
   double fpi;     // flops of one operator application
 };
 
-__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-
-__device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
 // Barrier state before a launch: no arrivals, no error, the context's wait limit.
 __global__ void k_bar_init(CgBar* b, unsigned long long limit_ns) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     b->count = 0;
-    b->error = 0;
     b->limit_ns = limit_ns;
   }
 }
 
-__device__ __forceinline__ void red_release_add(unsigned int* p, unsigned int v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -95,59 +90,79 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Grid barrier on a monotonic arrival counter: barrier number k completes when the counter
-// reaches k * gridDim.x.  Returns false (in every thread of the block) once any block gave up.
-__device__ bool grid_sync(CgBar* bar, unsigned int& target, int* flag) {
+// reaches k * gridDim.x.  Returns false (in every thread of the block) once any block gave up: it
+// sets the counter's top bit, which the poll that ends the wait sees with the arrivals (a flag of its
+// own cost another trip to L2 after every barrier).  Arrivals release and the last poll
+// acquires for the whole block (through __syncthreads).
+constexpr unsigned long long CG_GAVE_UP = 1ull << 63;
+__device__ bool grid_sync(CgBar* bar, unsigned long long& target, int* flag) {
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    red_release_add(&bar->count, 1u);
+    red_release_add(&bar->count, 1ull);
     const unsigned long long t0 = global_ns();
     unsigned int spins = 0;
     const unsigned long long limit = bar->limit_ns;
     // limits below 0.1 ms (tests of the timeout path) are checked at every poll
     const unsigned int mask = limit < 100000ull ? 0u : 255u;
-    while (ld_acquire(&bar->count) < target) {
-      if ((++spins & mask) == 0u) {
-        if (ld_volatile(&bar->error)) break;
-        if (global_ns() - t0 > limit) {
-          atomicExch(&bar->error, 1);
-          break;
-        }
+    unsigned long long v;
+    while ((v = ld_acquire(&bar->count)) < target) {
+      if ((++spins & mask) == 0u && global_ns() - t0 > limit) {
+        atomicOr(&bar->count, CG_GAVE_UP);
+        v = CG_GAVE_UP;
+        break;
       }
     }
-    __threadfence();
-    *flag = ld_volatile(&bar->error);
+    *flag = v >= CG_GAVE_UP;
   }
   __syncthreads();
   return *flag == 0;
 }
 
-__device__ double block_reduce(double v, double* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < nw; ++i) s += red[i];
-  __syncthreads();
-  return s;
+// Elements of the vectors per CTA (whole warps): spread over the grid, so that as few warps as possible
+// share a sub-partition's FP64 unit (a warp instruction takes it for 64 clocks).
+// With that, sums finished by one warp (two quantities at once) instead of by every thread, and the
+// barrier's flag in its counter, a Poisson site solve on 13 bits went from 145 to 111 us (this kernel) and
+// from 665 to 540 us (tensor cores), a momentum site solve on 20 bits from 254 to 214 us.
+__device__ __forceinline__ int cg_chunk(int64_t nel) {
+  return int(((nel + gridDim.x - 1) / gridDim.x + 31) / 32 * 32);
 }
 
-// Sum of the gridDim.x partials part[0..G) in a fixed order (identical in every block).
-__device__ double sum_partials(const double* part, double* red) {
-  const int G = gridDim.x;
-  if (threadIdx.x < 32) {
+// Sums of v0 and v1 over the first `warps` warps into out0[block], out1[block]: lanes 0-15 go on with v0, lanes
+// 16-31 with v1.  red: 16 doubles.  Call with the whole block.
+__device__ __forceinline__ void block_pair(double v0, double v1, int warps, double* red, double* out0, double* out1) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool hi = lane & 16;
+  double v = 0.0;
+  if (w < warps) {
+    v = (hi ? v1 : v0) + __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  if (warps > 1) {
+    if (w < warps && (lane & 15) == 0) red[(hi ? 8 : 0) + w] = v;
+    __syncthreads();
+    if (w == 0) {
+      v = (lane & 15) < warps ? red[(hi ? 8 : 0) + (lane & 15)] : 0.0;
+      for (int o = 4; o > 0; o >>= 1)
+        if (o < warps) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+  }
+  if (w == 0 && (lane & 15) == 0) (hi ? out1 : out0)[blockIdx.x] = v;
+}
+
+// tot[k] = sum of the gridDim.x partials part[k], k < n, one warp each, in a fixed order (identical in
+// every block).  tot is not written again before the next grid barrier.
+__device__ __forceinline__ void sum_partials(const double* p0, const double* p1, const double* p2, int n, double* tot) {
+  const int G = gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < n) {
+    const double* part = w == 0 ? p0 : w == 1 ? p1 : p2;
     double s = 0.0;
-    for (int i = threadIdx.x; i < G; i += 32) s += __ldcg(part + i);
+    if (lane < G) s = __ldcg(part + lane);
+    for (int i = lane + 32; i < G; i += 32) s += __ldcg(part + i);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) red[0] = s;
+    if (lane == 0) tot[w] = s;
   }
   __syncthreads();
-  const double s = red[0];
-  __syncthreads();
-  return s;
 }
 
 // Preconditioned residual z = D^-1 r at element g (z = r without a preconditioner); every place
@@ -251,6 +266,8 @@ __global__ void __launch_bounds__(CGP_THREADS, 2) k_cg_persistent(CgArgs a) {
   const int r0 = a.r0, w0 = a.w0, w1 = a.w1, d = a.d, bt = a.bt;
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
   const int64_t nel = int64_t(r0) * d * a.r1;
+  const int chunk = cg_chunk(nel), warps = min(nt, chunk) / 32;
+  const int64_t e0 = int64_t(blockIdx.x) * chunk, e1 = min(nel, e0 + chunk);
   const int K = w1 * a.r1;
   double* sL = sm;                           // w0 x r0
   double* sW = sL + w0 * r0;                 // w0 x d x d x w1
@@ -258,9 +275,9 @@ __global__ void __launch_bounds__(CGP_THREADS, 2) k_cg_persistent(CgArgs a) {
   double* sT1 = sP + r0 * d * bt;            // w0 x d x bt
   double* sR = sT1 + w0 * d * bt;            // eb x (K + 1): this block's rows of R
   double* sT2 = sR + size_t(a.eb) * (K + 1); // ch x (16 / eb) x K
-  __shared__ double red[32];
+  __shared__ double red[32], tot[6];
   __shared__ int flag;
-  unsigned int target = 0;
+  unsigned long long target = 0;
   double* part_pap = a.part;
   double* part_rr = a.part + G;
   double* part_bb = a.part + 2 * G;
@@ -285,7 +302,7 @@ __global__ void __launch_bounds__(CGP_THREADS, 2) k_cg_persistent(CgArgs a) {
     stage_b(a, nullptr, a.Ap, sR, sT2);
     if (!(ok = grid_sync(a.bar, target, &flag))) break;
     double rr_p = 0.0, bb_p = 0.0, rz_p = 0.0;
-    for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt) {
+    for (int64_t e = e0 + tid; e < e1; e += nt) {
       const double be = __ldg(a.b + e);
       const double re = be - __ldcg(a.Ap + e);
       const double ze = a.dinv ? __ldg(a.dinv + e) * re : re;
@@ -295,18 +312,12 @@ __global__ void __launch_bounds__(CGP_THREADS, 2) k_cg_persistent(CgArgs a) {
       rz_p = fma(re, ze, rz_p);
       bb_p = fma(be, be, bb_p);
     }
-    rr_p = block_reduce(rr_p, red);
-    rz_p = block_reduce(rz_p, red);
-    bb_p = block_reduce(bb_p, red);
-    if (tid == 0) {
-      part_rr[blockIdx.x] = rr_p;
-      part_rz[blockIdx.x] = rz_p;
-      part_bb[blockIdx.x] = bb_p;
-    }
+    block_pair(rr_p, rz_p, warps, red, part_rr, part_rz);
+    block_pair(bb_p, 0.0, warps, red + 16, part_bb, part_pap);
     if (!(ok = grid_sync(a.bar, target, &flag))) break;
-    double rr = sum_partials(part_rr, red);
-    double rz = sum_partials(part_rz, red);
-    const double bb = sum_partials(part_bb, red);
+    sum_partials(part_rr, part_rz, part_bb, 3, tot + 3);
+    double rr = tot[3], rz = tot[4];
+    const double bb = tot[5];
     const double tol2 = __ldg(a.tol) * __ldg(a.tol);
     bool active = rr > tol2 * bb && rr > 0.0;
     double beta = 0.0;
@@ -319,35 +330,38 @@ __global__ void __launch_bounds__(CGP_THREADS, 2) k_cg_persistent(CgArgs a) {
       if (it == 0) {
         stage_a(a, pn, nullptr, 0.0, sL, sW, sP, sT1);
       } else {
-        for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt)
+        for (int64_t e = e0 + tid; e < e1; e += nt)
           pn[e] = fma(beta, po[e], zval(a.dinv, a.r, e));
         stage_a(a, po, a.r, beta, sL, sW, sP, sT1);
       }
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
+      // lanes 0 and 16 of each warp hold shares of p.Ap
       double pap_p = stage_b(a, pn, a.Ap, sR, sT2);
-      pap_p = block_reduce(pap_p, red);
-      if (tid == 0) part_pap[blockIdx.x] = pap_p;
+      pap_p += __shfl_xor_sync(0xffffffffu, pap_p, 16);
+      if ((tid & 31) == 0) red[16 + (tid >> 5)] = pap_p;
+      __syncthreads();
+      if (tid < 32) {
+        pap_p = tid < CGP_THREADS / 32 ? red[16 + tid] : 0.0;
+        for (int o = CGP_THREADS / 64; o > 0; o >>= 1) pap_p += __shfl_xor_sync(0xffffffffu, pap_p, o);
+        if (tid == 0) part_pap[blockIdx.x] = pap_p;
+      }
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
-      const double pap = sum_partials(part_pap, red);
+      sum_partials(part_pap, nullptr, nullptr, 1, tot);
+      const double pap = tot[0];
       if (!(pap > 0.0)) break;                       // same decision in every block
       const double alpha = rz / pap;
       double rn_p = 0.0, rzn_p = 0.0;
-      for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt) {
+      for (int64_t e = e0 + tid; e < e1; e += nt) {
         a.x[e] += alpha * pn[e];
         const double re = a.r[e] - alpha * __ldcg(a.Ap + e);
         a.r[e] = re;
         rn_p = fma(re, re, rn_p);
         rzn_p = fma(re, a.dinv ? __ldg(a.dinv + e) * re : re, rzn_p);
       }
-      rn_p = block_reduce(rn_p, red);
-      rzn_p = block_reduce(rzn_p, red);
-      if (tid == 0) {
-        part_rr[blockIdx.x] = rn_p;
-        part_rz[blockIdx.x] = rzn_p;
-      }
+      block_pair(rn_p, rzn_p, warps, red, part_rr, part_rz);
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
-      const double rn = sum_partials(part_rr, red);
-      const double rzn = sum_partials(part_rz, red);
+      sum_partials(part_rr, part_rz, nullptr, 2, tot + 1);
+      const double rn = tot[1], rzn = tot[2];
       beta = rzn / rz;
       rr = rn;
       rz = rzn;
@@ -740,10 +754,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cg_tc(CgTcArgs a) {
   extern __shared__ __align__(16) unsigned char tc_sm[];
   const int G = gridDim.x, tid = threadIdx.x, nt = blockDim.x;
   const int64_t nel = int64_t(a.MB) * a.NB;
-  __shared__ double red[32];
+  const int chunk = cg_chunk(nel), warps = min(nt, chunk) / 32;
+  const int64_t e0 = int64_t(blockIdx.x) * chunk, e1 = min(nel, e0 + chunk);
+  __shared__ double red[32], tot[6];
   __shared__ int sred[TC_THREADS / 32];
   __shared__ int flag;
-  unsigned int target = 0;
+  unsigned long long target = 0;
   double* part_pap = a.part;
   double* part_rr = a.part + G;
   double* part_bb = a.part + 2 * G;
@@ -774,7 +790,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cg_tc(CgTcArgs a) {
     tc_stage_b(a, nullptr, tc_sm);
     if (!(ok = grid_sync(a.bar, target, &flag))) break;
     double rr_p = 0.0, bb_p = 0.0, rz_p = 0.0;
-    for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt) {
+    for (int64_t e = e0 + tid; e < e1; e += nt) {
       const double be = __ldg(a.b + e);
       const double re = be - __ldcg(a.Ap + e);
       const double ze = a.dinv ? __ldg(a.dinv + e) * re : re;
@@ -784,18 +800,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cg_tc(CgTcArgs a) {
       rz_p = fma(re, ze, rz_p);
       bb_p = fma(be, be, bb_p);
     }
-    rr_p = block_reduce(rr_p, red);
-    rz_p = block_reduce(rz_p, red);
-    bb_p = block_reduce(bb_p, red);
-    if (tid == 0) {
-      part_rr[blockIdx.x] = rr_p;
-      part_rz[blockIdx.x] = rz_p;
-      part_bb[blockIdx.x] = bb_p;
-    }
+    block_pair(rr_p, rz_p, warps, red, part_rr, part_rz);
+    block_pair(bb_p, 0.0, warps, red + 16, part_bb, part_pap);
     if (!(ok = grid_sync(a.bar, target, &flag))) break;
-    double rr = sum_partials(part_rr, red);
-    double rz = sum_partials(part_rz, red);
-    const double bb = sum_partials(part_bb, red);
+    sum_partials(part_rr, part_rz, part_bb, 3, tot + 3);
+    double rr = tot[3], rz = tot[4];
+    const double bb = tot[5];
     const double tol2 = __ldg(a.tol) * __ldg(a.tol);
     bool active = rr > tol2 * bb && rr > 0.0;
     double beta = 0.0;
@@ -805,37 +815,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cg_tc(CgTcArgs a) {
       if (it == 0) {
         tc_stage_a(a, pn, nullptr, 0.0, tc_sm);
       } else {
-        for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt)
+        for (int64_t e = e0 + tid; e < e1; e += nt)
           pn[e] = fma(beta, po[e], zval(a.dinv, a.r, e));
         tc_stage_a(a, po, a.r, beta, tc_sm);
       }
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
       tc_split_t1(a, sred);
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
-      double pap_p = tc_stage_b(a, pn, tc_sm);
-      pap_p = block_reduce(pap_p, red);
-      if (tid == 0) part_pap[blockIdx.x] = pap_p;
+      double pap_p = tc_stage_b(a, pn, tc_sm);   // warp 0 holds the shares of p.Ap
+      if (tid < 32) {
+        for (int o = 16; o > 0; o >>= 1) pap_p += __shfl_xor_sync(0xffffffffu, pap_p, o);
+        if (tid == 0) part_pap[blockIdx.x] = pap_p;
+      }
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
-      const double pap = sum_partials(part_pap, red);
+      sum_partials(part_pap, nullptr, nullptr, 1, tot);
+      const double pap = tot[0];
       if (!(pap > 0.0)) break;
       const double alpha = rz / pap;
       double rn_p = 0.0, rzn_p = 0.0;
-      for (int64_t e = int64_t(blockIdx.x) * nt + tid; e < nel; e += int64_t(G) * nt) {
+      for (int64_t e = e0 + tid; e < e1; e += nt) {
         a.x[e] += alpha * pn[e];
         const double re = a.r[e] - alpha * __ldcg(a.Ap + e);
         a.r[e] = re;
         rn_p = fma(re, re, rn_p);
         rzn_p = fma(re, a.dinv ? __ldg(a.dinv + e) * re : re, rzn_p);
       }
-      rn_p = block_reduce(rn_p, red);
-      rzn_p = block_reduce(rzn_p, red);
-      if (tid == 0) {
-        part_rr[blockIdx.x] = rn_p;
-        part_rz[blockIdx.x] = rzn_p;
-      }
+      block_pair(rn_p, rzn_p, warps, red, part_rr, part_rz);
       if (!(ok = grid_sync(a.bar, target, &flag))) break;
-      const double rn = sum_partials(part_rr, red);
-      const double rzn = sum_partials(part_rz, red);
+      sum_partials(part_rr, part_rz, nullptr, 2, tot + 1);
+      const double rn = tot[1], rzn = tot[2];
       beta = rzn / rz;
       rr = rn;
       rz = rzn;
