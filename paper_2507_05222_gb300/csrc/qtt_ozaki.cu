@@ -31,54 +31,72 @@ constexpr int OZ_BM = 128;         // rows of A per CTA (8 warps x 16)
 constexpr int OZ_BN = 32;          // columns of B per CTA (4 n8 tiles)
 constexpr int OZ_THREADS = 256;
 
-// Exponent of each row r of X (R rows of K values, strides sR, sK; batch stride sB):
-// ex[b R + r] = e with max_k |X_rk| 2^-e < 1/2 (0 for a zero row).  One warp per row.
-__global__ void k_oz_rowexp(int64_t batch, int64_t R, int64_t K, const double* __restrict__ X, int64_t sB, int64_t sR,
-                            int64_t sK, int* __restrict__ ex, const int* __restrict__ guard) {
+// An operand to split: R rows of K values per batch (strides sR, sK; batch stride sB), its row exponents
+// ex[b R + r] and digit slices out[((b S + s) R + r) Kp + k].
+struct OzOperand {
+  const double* X;
+  int64_t R, sB, sR, sK;
+  int* ex;
+  __nv_bfloat16* out;
+};
+
+// Both operands of a product go through one launch of each of the two kernels below, and indices are
+// 32-bit where the sizes allow (a 64-bit division per element cost more than the digits): launches
+// and divisions were a fifth of a Hadamard product at bond 64.
+// One launch of each instead of two took the 20-bit Hadamard product from 15.7 to 14.4 ms.
+
+// Exponent of each row r: ex[b R + r] = e with max_k |X_rk| 2^-e < 1/2 (0 for a zero row).  One warp
+// per row, A's rows first.
+__global__ void k_oz_rowexp(int64_t batch, int64_t K, OzOperand A, OzOperand B, const int* __restrict__ guard) {
   if (guard && *guard == 0) return;
-  const int64_t wid = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
+  int64_t wid = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  const bool first = wid < batch * A.R;
+  if (!first) wid -= batch * A.R;
+  const int64_t R = first ? A.R : B.R, sK = first ? A.sK : B.sK;
   if (wid >= batch * R) return;
   const int64_t b = wid / R, r = wid - b * R;
-  const double* x = X + b * sB + r * sR;
+  const double* x = first ? A.X + b * A.sB + r * A.sR : B.X + b * B.sB + r * B.sR;
   // largest exponent field of the row (integer operations only: the FP64 unit is slow here)
   int mx = 0;
+#pragma unroll 4
   for (int64_t k = lane; k < K; k += 32)
     mx = max(mx, int((static_cast<unsigned long long>(__double_as_longlong(x[k * sK])) >> 52) & 0x7ff));
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  mx = __reduce_max_sync(0xffffffffu, mx);
   // max |x| < 2^(mx - 1022), so e = mx - 1021 gives |x| 2^-e < 1/2 (rows of zeros and subnormals:
   // e = 0, their digits vanish -- an absolute error below 2^-1021)
-  if (lane == 0) ex[b * R + r] = mx > 0 ? mx - 1021 : 0;
+  if (lane == 0) (first ? A.ex : B.ex)[wid] = mx > 0 ? mx - 1021 : 0;
 }
 
 // The S digits of every element, by integer arithmetic on the FP64 bit pattern: the element
 // as a fixed-point integer F = round(x 2^(8S - e)) (|F| < 2^(8S-1)), then balanced base-256
 // digits from the least significant up, d = ((F + 128) mod 256) - 128, F = (F - d) / 256; what
-// is left is the most significant digit, |d_1| <= 128.  Written as
-// out[((b S + s) R + r) Kp + k] (digit s + 1, bf16; zero for K <= k < Kp).  Threads walk k
-// fastest when X is contiguous along k, else r fastest, so that the reads coalesce.
-__global__ void k_oz_digits(int64_t batch, int64_t R, int64_t K, int64_t Kp, const double* __restrict__ X, int64_t sB,
-                            int64_t sR, int64_t sK, const int* __restrict__ ex, __nv_bfloat16* __restrict__ out,
-                            const int* __restrict__ guard, int P) {
+// is left is the most significant digit, |d_1| <= 128 (bf16; zero for K <= k < Kp).  Threads walk k
+// fastest when X is contiguous along k, else r fastest, so that the reads coalesce.  I: index type.
+template <class I>
+__global__ void k_oz_digits(I batch, I K, I Kp, OzOperand A, OzOperand B, const int* __restrict__ guard, int P) {
   if (guard && *guard == 0) return;
-  const int64_t total = batch * R * Kp;
-  const bool kfast = (sK == 1) || (sR != 1);
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-    int64_t b, r, k;
-    if (kfast) {
-      k = i % Kp;
-      const int64_t br = i / Kp;
-      r = br % R;
+  const I ta = batch * I(A.R) * Kp, total = ta + batch * I(B.R) * Kp;
+  const I stride = I(gridDim.x) * I(blockDim.x);
+  for (I i0 = I(blockIdx.x) * I(blockDim.x) + I(threadIdx.x); i0 < total; i0 += stride) {
+    const bool first = i0 < ta;
+    const I i = first ? i0 : i0 - ta, R = I(first ? A.R : B.R);
+    const int64_t sR = first ? A.sR : B.sR, sK = first ? A.sK : B.sK;
+    I b, r, k;
+    if (sK == 1 || sR != 1) {
+      const I br = i / Kp;
+      k = i - br * Kp;
       b = br / R;
+      r = br - b * R;
     } else {
-      r = i % R;
-      const int64_t bk = i / R;
-      k = bk % Kp;
+      const I bk = i / R;
+      r = i - bk * R;
       b = bk / Kp;
+      k = bk - b * Kp;
     }
-    const long long F0 = (k < K) ? oz_fixed(X[b * sB + r * sR + k * sK], ex[b * R + r]) : 0;
-    long long F = F0;
-    __nv_bfloat16* o = out + ((b * OZ_S) * R + r) * Kp + k;
+    const double* X = first ? A.X + b * A.sB : B.X + b * B.sB;
+    long long F = k < K ? oz_fixed(X[r * sR + k * sK], (first ? A.ex : B.ex)[b * R + r]) : 0;
+    __nv_bfloat16* o = (first ? A.out : B.out) + ((int64_t(b) * OZ_S) * R + r) * Kp + k;
 #pragma unroll
     for (int s = OZ_S - 1; s >= 1; --s) {
       const long long dg = ((F + 128) & 255) - 128;
@@ -87,6 +105,18 @@ __global__ void k_oz_digits(int64_t batch, int64_t R, int64_t K, int64_t Kp, con
     }
     o[0] = __float2bfloat16_rn(float(F));   // |F| <= 128
   }
+}
+
+void oz_split(Ctx& c, int64_t batch, int64_t K, int64_t Kp, const OzOperand& A, const OzOperand& B, int P) {
+  const int64_t rows = batch * (A.R + B.R), total = rows * Kp;
+  k_oz_rowexp<<<unsigned((rows * 32 + 255) / 256), 256, 0, c.stream>>>(batch, K, A, B, c.guard);
+  after_launch(c, "oz_rowexp");
+  const unsigned blocks = unsigned(std::min<int64_t>((total + 255) / 256, 8192));
+  if (total <= (int64_t(1) << 31))   // i0 + stride stays below 2^32: the stride is at most 2^21
+    k_oz_digits<uint32_t><<<blocks, 256, 0, c.stream>>>(uint32_t(batch), uint32_t(K), uint32_t(Kp), A, B, c.guard, P);
+  else
+    k_oz_digits<int64_t><<<blocks, 256, 0, c.stream>>>(batch, K, Kp, A, B, c.guard, P);
+  after_launch(c, "oz_digits");
 }
 
 // C = alpha A B + beta C from the digit slices of A (rows) and of B (columns).  CTA tile
@@ -252,20 +282,7 @@ void gemm_ozaki(Ctx& c, int64_t batch, int64_t M, int64_t N, int64_t K, double a
   int* ea = reinterpret_cast<int*>(e.p);
   int* eb = ea + batch * M;
   ProfScope ps(c, KC_GEMM, 2.0 * double(batch) * double(M) * double(N) * double(K));
-  {
-    const int64_t wa = batch * M, wb = batch * N;
-    k_oz_rowexp<<<unsigned((wa * 32 + 255) / 256), 256, 0, c.stream>>>(batch, M, K, A, sAb, sAm, sAk, ea, c.guard);
-    after_launch(c, "oz_rowexp_a");
-    k_oz_rowexp<<<unsigned((wb * 32 + 255) / 256), 256, 0, c.stream>>>(batch, N, K, B, sBb, sBn, sBk, eb, c.guard);
-    after_launch(c, "oz_rowexp_b");
-    const int64_t ta = batch * M * Kp, tb = batch * N * Kp;
-    k_oz_digits<<<unsigned(std::min<int64_t>((ta + 255) / 256, 8192)), 256, 0, c.stream>>>(batch, M, K, Kp, A, sAb,
-                                                                                          sAm, sAk, ea, As, c.guard, P);
-    after_launch(c, "oz_digits_a");
-    k_oz_digits<<<unsigned(std::min<int64_t>((tb + 255) / 256, 8192)), 256, 0, c.stream>>>(batch, N, K, Kp, B, sBb,
-                                                                                          sBn, sBk, eb, Bs, c.guard, P);
-    after_launch(c, "oz_digits_b");
-  }
+  oz_split(c, batch, K, Kp, OzOperand{A, M, sAb, sAm, sAk, ea, As}, OzOperand{B, N, sBb, sBn, sBk, eb, Bs}, P);
   // Split K (in whole chunks) until the grid covers the SMs once: this kernel holds one CTA per
   // SM (its shared memory), and products such as (c s) x (e f) x d have few output tiles but a
   // long k.
@@ -302,12 +319,8 @@ void gemm_ozaki(Ctx& c, int64_t batch, int64_t M, int64_t N, int64_t K, double a
 // (K values each, strides sR, sK; zero digits for K <= k < Kp).
 void oz_split_rows(Ctx& c, int64_t R, int64_t K, int64_t Kp, const double* X, int64_t sR, int64_t sK, void* out,
                    int* ex) {
-  k_oz_rowexp<<<unsigned((R * 32 + 255) / 256), 256, 0, c.stream>>>(1, R, K, X, 0, sR, sK, ex, c.guard);
-  after_launch(c, "oz_rowexp");
-  const int64_t t = R * Kp;
-  k_oz_digits<<<unsigned(std::min<int64_t>((t + 255) / 256, 8192)), 256, 0, c.stream>>>(
-      1, R, K, Kp, X, 0, sR, sK, ex, static_cast<__nv_bfloat16*>(out), c.guard, OZ_S);
-  after_launch(c, "oz_digits");
+  oz_split(c, 1, K, Kp, OzOperand{X, R, 0, sR, sK, ex, static_cast<__nv_bfloat16*>(out)},
+           OzOperand{X, 0, 0, sR, sK, nullptr, nullptr}, OZ_S);
 }
 
 }  // namespace qtt
