@@ -24,23 +24,24 @@ constexpr float NN_B1 = 0.9f, NN_B2 = 0.999f, NN_EPS = 1e-8f;
 
 unsigned nn_blocks(int64_t n, int t) { return unsigned(std::min<int64_t>((n + t - 1) / t, 65535 * 8)); }
 
-// The convolution and its data gradient.  FLIP = false: out[n, o] = b[o] + sum_c w[o, c] * in[n, c]
+// The convolution and its data gradient, for large layers.  FLIP = false: out[n, o] = b[o] + sum_c w[o, c] * in[n, c]
 // (with ReLU, and the layer's input affine (x - shift[c]) scale[c], zero outside the grid in the
 // mapped values); FLIP = true: out[n, c] = sum_o w[o, c] (transposed stencil) in[n, o], zero where
 // the activation `act` of the layer below is not positive (its ReLU).  A CTA computes an R x 32
 // tile of pixels for 4 COT channels: a thread has four neighbouring pixels of COT channels in
 // registers, input rows and weights staged in shared memory CC input channels at a time, so that
 // 36 COT multiply-adds take 18 + 9 COT / 4 shared loads: the FP32 pipe bounds it, where one thread
-// per output loaded an input and a weight for each multiply-add.  The order of each output's sum is
+// per output (k_conv_direct) loads an input and a weight for each multiply-add.  The order of each output's sum is
 // unchanged (input channels, then taps).  With k_conv_wgrad a training step of 8 x 128 x 128 cells,
 // width 32, depth 4 (15 GFLOP) went from 14.4 to 1.02 ms.
-template <int COT, bool FLIP>
+template <bool FLIP>
 __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, const float* __restrict__ in,
                                               const float* __restrict__ shift, const float* __restrict__ scale,
                                               const float* __restrict__ w, const float* __restrict__ b,
                                               const float* __restrict__ act, float* __restrict__ out, int relu) {
+  constexpr int COT = 8;                         // output channels of a thread
   constexpr int CC = 4;                          // input channels per stage
-  constexpr int NG = COT == 1 ? 1 : 4;           // channel groups of a CTA
+  constexpr int NG = 4;                          // channel groups of a CTA
   constexpr int R = 256 / NG / 8;                // tile rows (8 threads of four pixels a row)
   constexpr int CO = COT * NG;
   __shared__ float xs[CC][R + 2][36];
@@ -94,20 +95,14 @@ __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, cons
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
           const int ra = FLIP ? 2 - a : a, re = FLIP ? 2 - e : e;
-          if (COT == 1) {
-            const float wv = ws[c][a * 3 + e][og];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[0][q] = fmaf(wv, x[ra][q + re], acc[0][q]);
-          } else {
+          for (int o = 0; o < COT; o += 4) {
+            const float4 wv = *reinterpret_cast<const float4*>(&ws[c][a * 3 + e][og * COT + o]);
+            const float wq[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
-            for (int o = 0; o < COT; o += 4) {
-              const float4 wv = *reinterpret_cast<const float4*>(&ws[c][a * 3 + e][og * COT + o]);
-              const float wq[4] = {wv.x, wv.y, wv.z, wv.w};
+            for (int u = 0; u < 4; ++u)
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[(o + u) % COT][q] = fmaf(wq[u], x[ra][q + re], acc[(o + u) % COT][q]);
-            }
+              for (int q = 0; q < 4; ++q) acc[o + u][q] = fmaf(wq[u], x[ra][q + re], acc[o + u][q]);
           }
         }
     }
@@ -128,6 +123,78 @@ __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, cons
       else if (relu) v = fmaxf(v, 0.f);
       out[g] = v;
     }
+  }
+}
+
+// The same with one thread per output, for small layers: a load for each multiply-add, but no stages, so
+// the time is that of one output's chain until the grid fills the chip.
+template <bool FLIP>
+__global__ void __launch_bounds__(256) k_conv_direct(int B, int ni, int no, int H, int W, const float* __restrict__ in,
+                                                     const float* __restrict__ shift, const float* __restrict__ scale,
+                                                     const float* __restrict__ w, const float* __restrict__ b,
+                                                     const float* __restrict__ act, float* __restrict__ out, int relu) {
+  const int64_t total = int64_t(B) * no * H * W, per = int64_t(H) * W;
+  for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < total; idx += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t plane = idx / per;
+    const int at = int(idx - plane * per), i = at / W, j = at - i * W;
+    const int n = int(plane / no), o = int(plane - int64_t(n) * no);
+    int jc[3];
+    jc[0] = j == 0 ? W - 1 : j - 1;
+    jc[1] = j;
+    jc[2] = j == W - 1 ? 0 : j + 1;
+    float s = FLIP ? 0.f : b[o];
+    for (int c = 0; c < ni; ++c) {
+      const float* xc = in + (int64_t(n) * ni + c) * per;
+      const float* wc = FLIP ? w + (int64_t(c) * no + o) * 9 : w + (int64_t(o) * ni + c) * 9;
+      const bool affine = !FLIP && shift;
+      const float sh = affine ? shift[c] : 0.f, sc = affine ? scale[c] : 1.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int ii = FLIP ? i - a + 1 : i + a - 1;
+        const bool inside = ii >= 0 && ii < H;
+        const float* row = xc + int64_t(inside ? ii : i) * W;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          float v = row[jc[FLIP ? 2 - e : e]];
+          if (affine) v = (v - sh) * sc;
+          s = inside ? fmaf(wc[a * 3 + e], v, s) : s;
+        }
+      }
+    }
+    if (FLIP) s = act[idx] > 0.f ? s : 0.f;
+    else if (relu) s = fmaxf(s, 0.f);
+    out[idx] = s;
+  }
+}
+
+// Weight and bias gradients of a small layer, one CTA per value: [0, co ci 9) the weights (o, c, a, e), then
+// the biases, written in that order.  Fixed summation order.
+__global__ void __launch_bounds__(256) k_conv_wgrad_direct(int B, int ci, int co, int H, int W, const float* __restrict__ x,
+                                                           const float* __restrict__ shift, const float* __restrict__ scale,
+                                                           const float* __restrict__ dy, float* __restrict__ grad) {
+  __shared__ float red[8];
+  const int nw = co * ci * 9, blk = blockIdx.x;
+  const bool bias = blk >= nw;
+  const int o = bias ? blk - nw : blk / (ci * 9), k = bias ? 0 : blk % (ci * 9), c = k / 9, a = (k % 9) / 3, e = k % 3;
+  const float sh = !bias && shift ? shift[c] : 0.f, sc = !bias && shift ? scale[c] : 1.f;
+  const int per = H * W, total = B * per;
+  float s = 0.f;
+  for (int t = threadIdx.x; t < total; t += 256) {
+    const int n = t / per, at = t - n * per, i = at / W, j = at - i * W;
+    const float g = dy[(int64_t(n) * co + o) * per + at];
+    const int ii = i + a - 1;
+    int jj = j + e - 1;
+    jj = jj < 0 ? jj + W : jj >= W ? jj - W : jj;
+    if (bias) s += g;
+    else if (ii >= 0 && ii < H) s = fmaf(g, (x[(int64_t(n) * ci + c) * per + int64_t(ii) * W + jj] - sh) * sc, s);
+  }
+  for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s = 0.f;
+    for (int q = 0; q < 8; ++q) s += red[q];
+    grad[blk] = s;
   }
 }
 
@@ -371,18 +438,25 @@ __global__ void k_moments(int64_t n, const float* __restrict__ x, double* __rest
   }
 }
 
-// Channels in groups of 32 (eight a thread) where the layer has more than four, else one a thread.
+// Direct up to 2^19 outputs and for at most four output channels (the tiled kernel has 32), tiled above.  us
+// a layer (mean over a network's), direct / tiled: 2 x 16 x 16 cells, width 32 13 / 31; 2 x 128 x 16, width 24
+// 12 / 25; 8 x 64 x 48, width 32 42 / 26; 8 x 64 x 64 59 / 30; 8 x 128 x 128 205 / 76.  One output channel:
+// 8 x 64 x 64 20 / 58.
+constexpr int64_t kConvDirect = int64_t(1) << 19;     // outputs
+// Direct up to 2^21 multiply-adds over at most 4096 pixels (16 a thread).  us a layer (mean over a network's),
+// direct / tiled with its sum: 32 x 16 cells, width 12 4.2 / 14.6; 4 x 32 x 48, width 16 40 / 15; 8 x 128 x 128,
+// width 32 3156 / 81.  A layer of one by 8 channels on 128 x 128 cells took 27 direct, its network's layers 11.5
+// tiled.
+constexpr int64_t kWgradDirect = int64_t(1) << 21, kWgradDirectPixels = 4096;
 template <bool FLIP>
 void conv(Ctx& c, int B, int ni, int no, int H, int W, const float* in, const float* shift, const float* scale,
           const float* w, const float* b, const float* act, float* out, int relu) {
-  const int R = no > 4 ? 8 : 32;
-  const int64_t tiles = int64_t(B) * ((W + 31) / 32) * ((H + R - 1) / R);
-  if (no > 4)
-    k_conv<8, FLIP><<<dim3(unsigned(tiles), unsigned((no + 31) / 32)), 256, 0, c.stream>>>(ni, no, H, W, in, shift, scale,
-                                                                                          w, b, act, out, relu);
+  const int64_t outputs = int64_t(B) * no * H * W, tiles = int64_t(B) * ((W + 31) / 32) * ((H + 7) / 8);
+  if (no <= 4 || outputs <= kConvDirect)
+    k_conv_direct<FLIP><<<nn_blocks(outputs, 256), 256, 0, c.stream>>>(B, ni, no, H, W, in, shift, scale, w, b, act, out, relu);
   else
-    k_conv<1, FLIP><<<dim3(unsigned(tiles), unsigned(no)), 256, 0, c.stream>>>(ni, no, H, W, in, shift, scale, w, b, act,
-                                                                              out, relu);
+    k_conv<FLIP><<<dim3(unsigned(tiles), unsigned((no + 31) / 32)), 256, 0, c.stream>>>(ni, no, H, W, in, shift, scale, w, b,
+                                                                                       act, out, relu);
   after_launch(c, FLIP ? "nn_conv_bwd_data" : "nn_conv_fwd");
 }
 
@@ -507,16 +581,22 @@ float Net::train_step(int B, int H, int W, const float* x, const float* y, float
     const float* in = k == 0 ? x : reinterpret_cast<float*>(acts[k - 1].p);
     float* dw = grad + offs[k];
     const int64_t nw = int64_t(co) * ci * 9 + co;
-    const int64_t tiles = int64_t(B) * ((W + CW_TC - 1) / CW_TC) * ((H + CW_TR - 1) / CW_TR);
-    const int chunks = ((co + CW_CH - 1) / CW_CH) * ((ci + CW_CH - 1) / CW_CH);
-    const int G = int(std::min<int64_t>(tiles, std::max(1, 2 * c.num_sms / chunks)));   // two CTAs per SM
-    DBuf wpart;
-    float* wp = fbuf(wpart, c, nw * G);
-    k_conv_wgrad<<<dim3(unsigned(G), unsigned(chunks)), 256, kWgradSmem, c.stream>>>(
-        B, ci, co, H, W, in, k == 0 ? shift : nullptr, k == 0 ? scale : nullptr, dy, wp);
-    after_launch(c, "nn_conv_wgrad");
-    k_conv_wsum<<<unsigned((nw * 8 + 255) / 256), 256, 0, c.stream>>>(nw, G, wp, dw);
-    after_launch(c, "nn_conv_wsum");
+    if (B * per <= kWgradDirectPixels && (nw - co) * B * per <= kWgradDirect) {
+      k_conv_wgrad_direct<<<unsigned(nw), 256, 0, c.stream>>>(B, ci, co, H, W, in, k == 0 ? shift : nullptr,
+                                                              k == 0 ? scale : nullptr, dy, dw);
+      after_launch(c, "nn_conv_wgrad");
+    } else {
+      const int64_t tiles = int64_t(B) * ((W + CW_TC - 1) / CW_TC) * ((H + CW_TR - 1) / CW_TR);
+      const int chunks = ((co + CW_CH - 1) / CW_CH) * ((ci + CW_CH - 1) / CW_CH);
+      const int G = int(std::min<int64_t>(tiles, std::max(1, 2 * c.num_sms / chunks)));   // two CTAs per SM
+      DBuf wpart;
+      float* wp = fbuf(wpart, c, nw * G);
+      k_conv_wgrad<<<dim3(unsigned(G), unsigned(chunks)), 256, kWgradSmem, c.stream>>>(
+          B, ci, co, H, W, in, k == 0 ? shift : nullptr, k == 0 ? scale : nullptr, dy, wp);
+      after_launch(c, "nn_conv_wgrad");
+      k_conv_wsum<<<unsigned((nw * 8 + 255) / 256), 256, 0, c.stream>>>(nw, G, wp, dw);
+      after_launch(c, "nn_conv_wsum");
+    }
     if (k > 0) {
       float* dx = fbuf(dxb, c, int64_t(B) * ci * per);
       conv<true>(c, B, co, ci, H, W, dy, nullptr, nullptr, params + offs[k], nullptr,
