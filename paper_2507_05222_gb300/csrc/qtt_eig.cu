@@ -20,7 +20,7 @@
 // (2 FMA a clock and SM: a product of order 128 takes 3.4 us of the whole chip) and by the grid
 // barrier (1.3 us) below n = 64.  The path that it replaces for these matrices (two-sided FP32
 // Jacobi of 1.5 us a round, levels three decades apart, some 35 launches a level; qtt_linalg.cu,
-// which stays for indefinite matrices and orders above 128) is measured against it at eigh_psd.
+// which stays for indefinite matrices and orders above 128) is measured against it at eigh_psd_fits.
 #include <algorithm>
 
 #include "qtt_algebra.h"
@@ -892,6 +892,9 @@ void eigh_psd_init_attributes() {
   g_psd_per_sm = per_sm;
 }
 
+// Orders 2 to 128, where the start's matrix fits a CTA's shared memory.  Against the general solver: a sketched
+// product at 20 bits (bond 64) 49.5 -> 23.5 ms, the encoding of 2^20 values 12.7 -> 3.2 ms; error against the
+// exact decomposition of the same product 4e-13 .. 3e-11 -> 2e-13 (12 inputs).
 bool eigh_psd_fits(int n, int m) {
   eigh_psd_init_attributes();
   return n >= 2 && n <= PS_MAX_N && m <= 256 && g_psd_per_sm >= 2;
