@@ -52,6 +52,9 @@ __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, cons
   const int n = blockIdx.x / (tw * th), t = blockIdx.x % (tw * th);
   const int i0 = (t / tw) * R, j0 = (t % tw) * 32, o0 = blockIdx.y * CO;
   const int64_t per = int64_t(H) * W;
+  // rows of the stencil that lie outside the grid are left out, not multiplied by zero: a weight that is
+  // not finite has no effect there (fmaxf would turn its NaN into a plausible 0)
+  const bool up = i0 + py > 0, down = i0 + py + 1 < H;
   float acc[COT][4];
 #pragma unroll
   for (int o = 0; o < COT; ++o) {
@@ -91,10 +94,12 @@ __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, cons
 #pragma unroll
         for (int q = 0; q < 6; ++q) x[a][q] = xs[c][py + a][4 * px + q];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+      for (int a = 0; a < 3; ++a) {
+        const int ra = FLIP ? 2 - a : a;
+        if ((ra == 0 && !up) || (ra == 2 && !down)) continue;
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
-          const int ra = FLIP ? 2 - a : a, re = FLIP ? 2 - e : e;
+          const int re = FLIP ? 2 - e : e;
 #pragma unroll
           for (int o = 0; o < COT; o += 4) {
             const float4 wv = *reinterpret_cast<const float4*>(&ws[c][a * 3 + e][og * COT + o]);
@@ -105,6 +110,7 @@ __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, cons
               for (int q = 0; q < 4; ++q) acc[o + u][q] = fmaf(wq[u], x[ra][q + re], acc[o + u][q]);
           }
         }
+      }
     }
   }
   const int i = i0 + py;
