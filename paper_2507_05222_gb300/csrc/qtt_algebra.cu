@@ -480,7 +480,10 @@ struct CutProj {
   bool trans = false;
 };
 
-// Eigenpairs of a cut's density matrix S (positive semidefinite; S = F^T F when F is given).
+// Eigenpairs of a cut's density matrix S (positive semidefinite; S = F^T F when F is given) for a cut
+// at keep: eigh_psd resolves pairs across that cut, not all pairs on one side of it.  A cut chosen
+// from the eigenvalues afterwards (a threshold) needs every pair and takes eigh: between singular values
+// 1e-5 apart eigh_psd left the truncated matrix 2e-4 off where eigh is exact to 1e-12.
 static void density_eigh(Ctx& c, int n, const double* S, double* w, double* V, int keep, const double* F = nullptr,
                          int m = 0) {
   if (eigh_psd_fits(n, m)) eigh_psd(c, n, S, w, V, keep, F, m);
@@ -560,7 +563,9 @@ qtt_mps* round_gram(Ctx& c, const qtt_mps* y, int chi, double eps) {
       DBuf T1(&c, size_t(a0) * nv), rho(&c, size_t(nv) * nv), w(&c, size_t(nv)), V(&c, size_t(nv) * nv);
       einsum(c, "aA,asc->Asc", 1.0, tv(G[k].p, {a0, a0}), tv(Z.p, {a0, d, c1}), 0.0, tv(T1.p, {a0, d, c1}));
       einsum(c, "Asc,AtD->sctD", 1.0, tv(T1.p, {a0, d, c1}), tv(Z.p, {a0, d, c1}), 0.0, tv(rho.p, {d, c1, d, c1}));
-      density_eigh(c, nv, rho.p, w.p, V.p, std::min(std::min(chi, m[k]), nv));
+      const int keep = std::min(std::min(chi, m[k]), nv);
+      if (fixed) density_eigh(c, nv, rho.p, w.p, V.p, keep);
+      else eigh(c, nv, rho.p, w.p, V.p, keep);
       int bk = choose_rank(c, w.p, nv, chi, eps, std::min(m[k], nv));
       add_discarded(c, rho.p, w.p, nv, bk);
       if (!z) out[k].reset(&c, size_t(bk) * nv);
