@@ -1161,9 +1161,8 @@ qtt_mps* zipup_hadamard(Ctx& c, const qtt_mps* a, const qtt_mps* b, int chi) {
 
 // ------------------------------------------------------------------ inner products, norms
 
-void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev) {
-  QTT_CHECK_ARG(a->n == b->n && a->d == b->d, "dot: shape mismatch");
-  if (dot_fused(c, a, b, out_dev)) return;
+// Site by site, two products each.
+static void dot_sites(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev) {
   const int n = a->n, d = a->d;
   DBuf E(&c, 1);
   fill(c, E.p, 1, 1.0);
@@ -1176,6 +1175,24 @@ void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev) {
     E = std::move(En);
   }
   copy(c, out_dev, E.p, 1);
+}
+
+// The value on the host (synchronises).  It does not depend on the wait limit: where a barrier of the fused
+// kernel's grid variant ran out, the overlap is computed again site by site, without waits.
+double dot_host(Ctx& c, const qtt_mps* a, const qtt_mps* b) {
+  QTT_CHECK_ARG(a->n == b->n && a->d == b->d, "dot: shape mismatch");
+  DBuf out(&c, 2);
+  double v[2] = {0.0, 1.0};
+  if (dot_fused(c, a, b, out.p)) {
+    QTT_CUDA(cudaMemcpyAsync(v, out.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+    QTT_CUDA(cudaStreamSynchronize(c.stream));
+  }
+  if (v[1] != 0.0) {
+    dot_sites(c, a, b, out.p);
+    QTT_CUDA(cudaMemcpyAsync(v, out.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+    QTT_CUDA(cudaStreamSynchronize(c.stream));
+  }
+  return v[0];
 }
 
 // ------------------------------------------------------------------ dense encode / decode

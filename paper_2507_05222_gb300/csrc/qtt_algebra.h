@@ -114,8 +114,9 @@ bool cg_team_fits(int r0, int r1, int w0, int w1, int d);
 void cg_team(Ctx& c, const double* L, const double* W, const double* R, const double* b, const double* xin, double* xout,
              int r0, int r1, int w0, int w1, int d, int iters, const double* tol_dev, int* total_dev);
 
-void dot_dev(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev);
-// The same in one launch (qtt_dot.cu); false if the bonds are beyond what it takes.
+double dot_host(Ctx& c, const qtt_mps* a, const qtt_mps* b);   // synchronises
+// In one launch (qtt_dot.cu): the value, and 1 instead of 0 if a wait ran out, to out_dev[0], out_dev[1];
+// false if the bonds are beyond what it takes.
 bool dot_fused(Ctx& c, const qtt_mps* a, const qtt_mps* b, double* out_dev);
 void sqrt_dev(Ctx& c, const double* in, double* out);
 qtt_mps* encode_dense(Ctx& c, const double* dense_dev, int n, int d, int chi, double eps);

@@ -122,15 +122,11 @@ void fill_info(Ctx& c, const qtt_mps* y, qtt_round_info* info, const DiscScope* 
   int mb = 1;
   for (int b : y->bonds) mb = std::max(mb, b);
   info->max_bond = mb;
-  DBuf d(&c, 1);
-  dot_dev(c, y, y, d.p);
-  double v[2] = {0.0, -1.0};
-  QTT_CUDA(cudaMemcpyAsync(&v[0], d.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+  double w = -1.0;
   if (disc && disc->acc.p)
-    QTT_CUDA(cudaMemcpyAsync(&v[1], disc->acc.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-  QTT_CUDA(cudaStreamSynchronize(c.stream));
-  info->norm = std::sqrt(std::max(v[0], 0.0));
-  info->discarded_norm = v[1] >= 0.0 ? std::sqrt(v[1]) : -1.0;
+    QTT_CUDA(cudaMemcpyAsync(&w, disc->acc.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+  info->norm = std::sqrt(std::max(dot_host(c, y, y), 0.0));
+  info->discarded_norm = w >= 0.0 ? std::sqrt(w) : -1.0;
 }
 
 __global__ void k_reorder(const double* __restrict__ src, double* __restrict__ dst, int ne, int nx, int ordering,
@@ -688,10 +684,7 @@ int mps_dot(qtt_ctx* ctx, const qtt_mps* a, const qtt_mps* b, double* out_host) 
   check_mps(b, "dot b");
   QTT_CHECK_ARG(a->n == b->n && a->d == b->d, "dot: a and b differ in n or d");
   Ctx& c = *reinterpret_cast<Ctx*>(ctx);
-  DBuf d(&c, 1);
-  dot_dev(c, a, b, d.p);
-  QTT_CUDA(cudaMemcpyAsync(out_host, d.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-  QTT_CUDA(cudaStreamSynchronize(c.stream));
+  *out_host = dot_host(c, a, b);
   API_END
 }
 

@@ -36,8 +36,8 @@ struct DotArgs {
   const double* B;
   double* ws;           // per side: E, E', T
   int64_t es, ts;       // sizes of E and T
-  double* out;
-  unsigned int* bar;    // grid variant: arrivals, error flag
+  double* out;          // the value; 0, or 1 where the grid variant gave up waiting
+  unsigned int* bar;    // grid variant: arrivals, whether a CTA gave up
   unsigned long long limit_ns;
 };
 
@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(DT_THREADS) k_dot_fused(const __grid_constant_
   if (tid == 0) {
     double v = 0.0;
     for (int w = 0; w < DT_THREADS / 32; ++w) v += red[w];
-    *a.out = ok ? v : __longlong_as_double(0x7ff8000000000000ll);
+    a.out[0] = v;
+    a.out[1] = ok ? 0.0 : 1.0;
   }
 }
 
