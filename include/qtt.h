@@ -193,8 +193,8 @@ int qtt_ctx_profile_phases(qtt_ctx* ctx, double* ms_out, int64_t* launches_out);
  * context still usable.  Takes effect for work enqueued afterwards (a captured step keeps the
  * limit it was captured with: set it before the first fractional_step or after
  * qtt_case_use_graph).  Tests shorten it to exercise the timeout path without any fault.
- * The values of overlaps do not depend on the limit: where a wait of the one-kernel overlap runs out, it
- * is computed again without waits. */
+ * The values of overlaps and of the roundings' eigenproblems do not depend on the limit: where a wait
+ * of the one-kernel overlap or of the eigensolver's grid runs out, the work is done again without waits. */
 int qtt_ctx_set_wait_limit(qtt_ctx* ctx, double seconds);
 /* How ALS local systems are solved (Sec. II.A.4).  Mode 2 runs each local CG solve as one
  * cooperative kernel on the FP64 pipe (one CTA per SM, grid barriers between its stages) where

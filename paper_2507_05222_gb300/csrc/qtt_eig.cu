@@ -38,8 +38,8 @@ constexpr float PS_DONE = 1e-3f;        // a sweep that met no larger cosine is 
 
 // Barrier and result record of one eigenproblem (device memory, set up by its start kernels).
 struct PsdState {
-  unsigned int count;
-  int error;
+  unsigned int count;      // arrivals at the level's barriers; top bit: a CTA gave up waiting
+  unsigned int left;       // CTAs that left the level because of that
   unsigned long long limit_ns;
   int t0, need;            // the next level's tail block and whether it is taken
   int e;                   // the matrix is worked on as S 2^-e
@@ -313,8 +313,8 @@ __global__ void __launch_bounds__(PS_THREADS) k_psd_start(int nfull, const doubl
       st->anorm = sqrt(double(f));
     }
     st->limit_ns = limit_ns;
-    st->error = 0;
     st->count = 0;
+    st->left = 0;
   }
   // Pivoted Cholesky, left-looking: the pivot's column is formed when it is chosen (four lanes a
   // row share the sum over the earlier columns), only the diagonal is kept up to date.  Every
@@ -525,27 +525,33 @@ __device__ __forceinline__ unsigned long long pr_ns() {
   return t;
 }
 
-// Grid barrier on a monotonic arrival counter, bounded by the context's wait limit (see qtt_cg.cu).
-__device__ bool pr_sync(PsdState* st, unsigned int& target, int* flag) {
-  target += gridDim.x;
+// Grid barrier on a monotonic arrival counter, bounded by the context's wait limit (see qtt_cg.cu).  A CTA
+// gives up by a compare-and-swap on a count that is not complete yet, so that the last barrier is passed by
+// every CTA or by none: a level that ran out of time has not touched what it started from.
+constexpr unsigned int PR_GAVE_UP = 1u << 31;
+struct PsdGrid {
+  int G, b;      // CTAs that share the level, this CTA's index among them
+};
+__device__ bool pr_sync(PsdState* st, const PsdGrid& g, unsigned int& target, int* flag) {
+  if (g.G == 1) {
+    __threadfence();
+    __syncthreads();
+    return true;
+  }
+  target += g.G;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&st->count), "r"(1u) : "memory");
     const unsigned long long t0 = pr_ns(), limit = st->limit_ns;
     const unsigned int mask = limit < 100000ull ? 0u : 255u;
-    unsigned int spins = 0;
-    while (pr_ld_acquire(&st->count) < target) {
-      if ((++spins & mask) == 0u) {
-        if (*reinterpret_cast<const volatile int*>(&st->error)) break;
-        if (pr_ns() - t0 > limit) {
-          atomicExch(&st->error, 1);
-          break;
-        }
-      }
+    unsigned int spins = 0, v;
+    while ((v = pr_ld_acquire(&st->count)) < target) {
+      if ((++spins & mask) == 0u && pr_ns() - t0 > limit && atomicCAS(&st->count, v, v | PR_GAVE_UP) == v) v |= PR_GAVE_UP;
+      if (v & PR_GAVE_UP) break;
     }
     __threadfence();
-    *flag = *reinterpret_cast<const volatile int*>(&st->error);
+    *flag = (v & PR_GAVE_UP) != 0u;
   }
   __syncthreads();
   return *flag == 0;
@@ -610,14 +616,14 @@ __device__ __forceinline__ long long pr_key(double v) {
 // given, T = L R with L (M x n, row-major) and R (n x n): the tiles of both dealt to the CTAs.
 // Sum of squares of (delta_ij - P_ij) (of_identity) or of the off-diagonal P_ij, all and (tail) those
 // with a column at t0 or beyond.
-__device__ float pr_products(int n, const double* U, const double* W, int K, double* P, bool of_identity,
-                             const double* L, const double* R, int M, double* T, int t0, float& tail, double* sA,
-                             double* sB) {
+__device__ float pr_products(const PsdGrid& g, int n, const double* U, const double* W, int K, double* P,
+                             bool of_identity, const double* L, const double* R, int M, double* T, int t0, float& tail,
+                             double* sA, double* sB) {
   const int nt = (n + PR_T - 1) / PR_T, sym = nt * (nt + 1) / 2, mt = T ? (M + PR_T - 1) / PR_T : 0;
   float nrm = 0.f;
   tail = 0.f;
   const int tid = threadIdx.x, l = tid & 3, oi = (tid >> 2) >> 3, oj = (tid >> 2) & 7;
-  for (int t = blockIdx.x; t < sym + mt * nt; t += gridDim.x) {
+  for (int t = g.b; t < sym + mt * nt; t += g.G) {
     if (t < sym) {
       int a = 0, r = t;
       while (r >= nt - a) { r -= nt - a; ++a; }
@@ -641,11 +647,11 @@ __device__ float pr_products(int n, const double* U, const double* W, int K, dou
 }
 
 // Xo[:, col(j)] = X + X E (mode 0), X (3 I - E) / 2 (mode 1), X E (mode 2); rank: column map or null.
-__device__ void pr_update(int n, const double* X, const double* E, double* Xo, int mode, const int* rank, double* sA,
-                          double* sB) {
+__device__ void pr_update(const PsdGrid& g, int n, const double* X, const double* E, double* Xo, int mode,
+                          const int* rank, double* sA, double* sB) {
   const int nt = (n + PR_T - 1) / PR_T;
   const int tid = threadIdx.x, l = tid & 3, oi = (tid >> 2) >> 3, oj = (tid >> 2) & 7;
-  for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
+  for (int t = g.b; t < nt * nt; t += g.G) {
     const int a = t / nt, b = t % nt, i = a * PR_T + oi, j = b * PR_T + oj;
     double s = pr_tile(X, n, false, a * PR_T, n, E, n, b * PR_T, n, n, sA, sB);
     if (l == 0 && i < n && j < n) {
@@ -656,11 +662,11 @@ __device__ void pr_update(int n, const double* X, const double* E, double* Xo, i
   }
 }
 
-__global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
+// One level by the CTAs of g; false, with V, w, lam and SXs as they were, if a wait ran out.
+__device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
   extern __shared__ __align__(16) double pr_sm[];
   PsdState* st = a.st;
-  if (a.level > 0 && st->need == 0) return;
-  const int n = a.n, tid = threadIdx.x, G = gridDim.x;
+  const int n = a.n, tid = threadIdx.x, G = g.G;
   const int Kmax = max(n, a.m);
   double* sA = pr_sm;
   double* sB = sA + PR_T * (Kmax + 2);
@@ -701,53 +707,53 @@ __global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
   };
   auto xtsx1 = [&]() {   // G = X^T X and B = F X or S X
     float tl;
-    const float v = pr_products(n, X, X, n, a.G, true, a.F ? a.F : a.S, X, a.F ? a.m : n, a.B, t0, tl, sA, sB);
+    const float v = pr_products(g, n, X, X, n, a.G, true, a.F ? a.F : a.S, X, a.F ? a.m : n, a.B, t0, tl, sA, sB);
     const float s = pr_block_sum(v, redf);
-    if (tid == 0) a.part[blockIdx.x] = s;
+    if (tid == 0) a.part[g.b] = s;
   };
   auto xtsx2 = [&]() {                  // SX = B^T B or X^T B
     float tl;
-    const float v = pr_products(n, a.F ? a.B : X, a.B, a.F ? a.m : n, a.SX, false, nullptr, nullptr, 0, nullptr, t0, tl,
+    const float v = pr_products(g, n, a.F ? a.B : X, a.B, a.F ? a.m : n, a.SX, false, nullptr, nullptr, 0, nullptr, t0, tl,
                                 sA, sB);
     const float s = pr_block_sum(v, redf);
     const float st_ = pr_block_sum(tl, redf);
     if (tid == 0) {
-      a.part[G + blockIdx.x] = s;
-      a.part[3 * G + blockIdx.x] = st_;
+      a.part[G + g.b] = s;
+      a.part[3 * G + g.b] = st_;
     }
   };
   do {
     // ---- the level's start: X = Y, or X = V diag(I, Y)
     const int nt0 = n - t0;
     if (a.level == 0) {
-      for (int e = blockIdx.x * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) X[e] = a.Y[e];
+      for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) X[e] = a.Y[e];
     } else {
-      for (int e = blockIdx.x * PR_THREADS + tid; e < n * t0; e += G * PR_THREADS) {
+      for (int e = g.b * PR_THREADS + tid; e < n * t0; e += G * PR_THREADS) {
         const int i = e / t0, j = e % t0;
         X[size_t(i) * n + j] = a.V[size_t(i) * n + j];
       }
       const int rt = (n + PR_T - 1) / PR_T, ct = (nt0 + PR_T - 1) / PR_T;
       const int l = tid & 3, oi = (tid >> 2) >> 3, oj = (tid >> 2) & 7;
-      for (int t = blockIdx.x; t < rt * ct; t += G) {
+      for (int t = g.b; t < rt * ct; t += G) {
         const int i0 = (t / ct) * PR_T, j0 = (t % ct) * PR_T;
         const double s = pr_tile(a.V + t0, n, false, i0, n, a.Y, nt0, j0, nt0, nt0, sA, sB);
         if (l == 0 && i0 + oi < n && j0 + oj < nt0) X[size_t(i0 + oi) * n + t0 + j0 + oj] = s;
       }
     }
-    if (!(ok = pr_sync(st, target, &flag))) break;
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
     // ---- Newton-Schulz
-    pr_products(n, X, X, n, a.G, true, nullptr, nullptr, 0, nullptr, n, unused, sA, sB);
-    if (!(ok = pr_sync(st, target, &flag))) break;
-    pr_update(n, X, a.G, Xn, 1, nullptr, sA, sB);
+    pr_products(g, n, X, X, n, a.G, true, nullptr, nullptr, 0, nullptr, n, unused, sA, sB);
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
+    pr_update(g, n, X, a.G, Xn, 1, nullptr, sA, sB);
     swap();
-    if (!(ok = pr_sync(st, target, &flag))) break;
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
     // ---- Ogita-Aishima iterations
     float before = 1.f;
     for (int it = 0; it < PR_MAX_IT; ++it) {
       xtsx1();
-      if (!(ok = pr_sync(st, target, &flag))) break;
+      if (!(ok = pr_sync(st, g, target, &flag))) break;
       xtsx2();
-      if (!(ok = pr_sync(st, target, &flag))) break;
+      if (!(ok = pr_sync(st, g, target, &flag))) break;
       lambda();
       if (tid < 32) {
         float ro = 0.f, so = 0.f, tl = 0.f;
@@ -778,7 +784,7 @@ __global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
       const int below = __syncthreads_count(tid < n && fi_ < tail_s);
       const float tail = (tail_s > 0.f && below >= 2 && n - below < a.keep) ? tail_s : 0.f;
       float big = 0.f;
-      for (int e = blockIdx.x * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) {
+      for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) {
         const int i = e / n, j = e % n;
         const double r = (i == j ? 1.0 : 0.0) - __ldcg(a.G + e);
         double v = 0.5 * r;
@@ -806,16 +812,16 @@ __global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
       __syncthreads();
       if (tid == 0) {
         for (int w = 1; w < PR_THREADS / 32; ++w) big = fmaxf(big, redf[w]);
-        a.part[2 * G + blockIdx.x] = big;
+        a.part[2 * G + g.b] = big;
       }
-      if (!(ok = pr_sync(st, target, &flag))) break;
-      pr_update(n, X, a.E, Xn, 0, nullptr, sA, sB);
+      if (!(ok = pr_sync(st, g, target, &flag))) break;
+      pr_update(g, n, X, a.E, Xn, 0, nullptr, sA, sB);
       swap();
       // the same decision in every CTA: the largest correction of this iteration
       float mb = 0.f;
       for (int i = tid & 31; i < G; i += 32) mb = fmaxf(mb, __ldcg(a.part + 2 * G + i));
       for (int o = 16; o > 0; o >>= 1) mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-      if (!(ok = pr_sync(st, target, &flag))) break;
+      if (!(ok = pr_sync(st, g, target, &flag))) break;
       // corrections shrink quadratically where the gaps resolve a pair, by a constant factor while a
       // cluster next to it is unresolved: mb^2 / before bounds the next one either way; a level at
       // its rounding floor no longer shrinks
@@ -824,32 +830,44 @@ __global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
     }
     if (!ok) break;
     // ---- Newton-Schulz, eigenvalues, and a last Newton-Schulz step into the sorted V
-    pr_products(n, X, X, n, a.G, true, nullptr, nullptr, 0, nullptr, n, unused, sA, sB);
-    if (!(ok = pr_sync(st, target, &flag))) break;
-    pr_update(n, X, a.G, Xn, 1, nullptr, sA, sB);
+    pr_products(g, n, X, X, n, a.G, true, nullptr, nullptr, 0, nullptr, n, unused, sA, sB);
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
+    pr_update(g, n, X, a.G, Xn, 1, nullptr, sA, sB);
     swap();
-    if (!(ok = pr_sync(st, target, &flag))) break;
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
     xtsx1();
-    if (!(ok = pr_sync(st, target, &flag))) break;
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
     xtsx2();
-    if (!(ok = pr_sync(st, target, &flag))) break;
+    if (!(ok = pr_sync(st, g, target, &flag))) break;
     lambda();
-    pr_update(n, X, a.G, a.V, 1, rank, sA, sB);
+    pr_update(g, n, X, a.G, a.V, 1, rank, sA, sB);
     if (a.tau_next > 0.0)
-      for (int e = blockIdx.x * PR_THREADS + tid; e < n * n; e += G * PR_THREADS)
+      for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS)
         a.SXs[size_t(rank[e / n]) * n + rank[e % n]] = __ldcg(a.SX + e);
-    if (blockIdx.x == 0) {
+    if (g.b == 0) {
       for (int i = tid; i < n; i += PR_THREADS) {
         a.lam[rank[i]] = sl[i];
         a.w[rank[i]] = ldexp(sl[i], st->e);
       }
     }
   } while (false);
-  if (!ok) {   // a barrier ran out: no result
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    for (int e = blockIdx.x * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) a.V[e] = nan;
-    if (blockIdx.x == 0)
-      for (int i = tid; i < n; i += PR_THREADS) a.w[i] = nan;
+  return ok;
+}
+
+// A level whose waits ran out is done again by the last CTA to leave it, alone and without waits, so that the
+// results do not depend on the wait limit (slow: one SM's FP64 units; not needed while the grid is resident).
+__global__ void __launch_bounds__(PR_THREADS, 2) k_psd_refine(PsdArgs a) {
+  __shared__ unsigned int before;
+  if (a.level > 0 && a.st->need == 0) return;
+  PsdGrid g = {int(gridDim.x), int(blockIdx.x)};
+  while (!psd_level(a, g)) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) before = atomicAdd(&a.st->left, 1u);
+    __syncthreads();
+    if (before != gridDim.x - 1) return;
+    __threadfence();
+    g = {1, 0};
   }
 }
 
@@ -863,7 +881,7 @@ __global__ void k_psd_tail(int n, int keep, double tau, const double* __restrict
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (threadIdx.x == 0) {
     st->t0 = n - c;
-    st->need = (c >= 2 && n - c < keep && st->error == 0) ? 1 : 0;
+    st->need = (c >= 2 && n - c < keep) ? 1 : 0;
   }
 }
 

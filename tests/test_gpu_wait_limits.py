@@ -32,3 +32,43 @@ def test_dot_does_not_depend_on_the_limit(ctx, n, d, bond):
         ctx.set_wait_limit(limit)
         for _ in range(3):
             assert abs(qtt.mps_dot(ctx, ga, gb) - tt.dot(a, b)) <= tol
+
+
+def matrix(N, chi, decades, seed):
+    """A matrix of singular values over the given decades and its best approximation of rank chi."""
+    g = inputs.rng(seed)
+    U, _ = np.linalg.qr(g.standard_normal((N, N)))
+    V, _ = np.linalg.qr(g.standard_normal((N, N)))
+    s = 10.0 ** (-decades * np.arange(N) / max(N - 1, 1))
+    return (U * s) @ V.T, (U[:, :chi] * s[:chi]) @ V[:, :chi].T
+
+
+@pytest.mark.parametrize("N,chi", [(2, 1), (9, 4), (33, 16), (64, 30), (128, 64)])
+def test_encode_does_not_depend_on_the_limit(ctx, N, chi):
+    """One truncating cut through its density matrix; bound as in test_gpu_psd_eig (1e-10)."""
+    from paper_2507_05222_gb300 import qtt
+    A, best = matrix(N, chi, 4.0, N)
+    for limit in (2.0, 1e-9, 2.0):
+        ctx.set_wait_limit(limit)
+        info = {}
+        v = qtt.qtt_decode(ctx, qtt.qtt_encode(ctx, A.ravel(), 2, chi, d=N, out_info=info)).reshape(N, N)
+        assert np.linalg.norm(v - best) <= 1e-10 * np.linalg.norm(best)
+        assert abs(info["norm"] - np.linalg.norm(best)) <= 1e-10 * np.linalg.norm(best)
+
+
+@pytest.mark.parametrize("h,chi,decades", [(4, 12, 4.0), (5, 17, 14.0), (6, 40, 14.0)])
+def test_sketched_product_does_not_depend_on_the_limit(ctx, h, chi, decades):
+    """The factored form, whose levels go on to the end of fourteen decades; bound as in
+    test_gpu_psd_eig (1e-11)."""
+    from paper_2507_05222_gb300 import qtt
+    N = 2 ** h
+    A, best = matrix(N, chi, decades, 7 * N)
+    x = [np.eye(2 ** (k + 1)).reshape(2 ** k, 2, 2 ** (k + 1)) for k in range(h)]
+    x.append(A.reshape(N, 2, N // 2))
+    x += [np.eye(2 ** k).reshape(2 ** k, 2, 2 ** (k - 1)) for k in range(h - 1, 0, -1)]
+    M = [np.eye(2).reshape(1, 2, 2, 1)] * (2 * h)
+    gM, gx = qtt.MPO.from_cores(ctx, M), qtt.MPS.from_cores(ctx, x)
+    for limit in (1e-9, 2.0):
+        ctx.set_wait_limit(limit)
+        v = qtt.qtt_decode(ctx, qtt.mpo_apply_round(ctx, gM, gx, chi, apply="sketch")).reshape(N, N)
+        assert np.linalg.norm(v - best) <= 1e-11 * np.linalg.norm(best)
