@@ -44,7 +44,7 @@ struct PsdState {
   int t0, need;            // the next level's tail block and whether it is taken
   int e;                   // the matrix is worked on as S 2^-e
   int pad;
-  double anorm;            // ||S 2^-e||_F (a threshold, FP32 accuracy)
+  double anorm;            // ||S 2^-e||_F, from level 0's refinement
 };
 
 __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
@@ -262,7 +262,6 @@ __global__ void __launch_bounds__(PS_THREADS) k_psd_start(int nfull, const doubl
   float* vi = vd + PS_MAX_N;
   int* order = reinterpret_cast<int*>(vi + PS_MAX_N);
   __shared__ double red[PS_THREADS / 32];
-  __shared__ float redf[PS_THREADS / 32];
   __shared__ int es;
   __shared__ unsigned int worst;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
@@ -287,13 +286,11 @@ __global__ void __launch_bounds__(PS_THREADS) k_psd_start(int nfull, const doubl
   }
   __syncthreads();
   const int e0 = es;
-  float fro = 0.f;
   for (int e = tid; e < n * n; e += PS_THREADS) {
     const int i = e / n, k = e % n;
     const double v = ldexp(S[size_t(i + t0) * nfull + (k + t0)], -e0);
     if (level == 0) Ssc[size_t(i) * nfull + k] = v;
     const float h = float(v), lo = float(v - double(h));
-    fro = fmaf(h, h, fro);
     if (k <= i) {
       Sh[ps_tri(i, k)] = h;
       Sl[ps_tri(i, k)] = lo;
@@ -301,17 +298,10 @@ __global__ void __launch_bounds__(PS_THREADS) k_psd_start(int nfull, const doubl
     }
   }
   for (int i = n + tid; i < PS_MAX_N; i += PS_THREADS) dh[i] = 0.f;
-  for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
-  if (tx == 0) redf[ty] = fro;
   for (int e = tid; e < nc * ld; e += PS_THREADS) A[e] = 0.f;
   __syncthreads();
   if (tid == 0) {
-    if (level == 0) {
-      float f = 0.f;
-      for (int w = 0; w < PS_THREADS / 32; ++w) f += redf[w];
-      st->e = e0;
-      st->anorm = sqrt(double(f));
-    }
+    if (level == 0) st->e = e0;
     st->limit_ns = limit_ns;
     st->count = 0;
     st->left = 0;
@@ -509,7 +499,9 @@ struct PsdArgs {
   double* w;            // eigenvalues (unscaled)
   double* lam;          // eigenvalues of the scaled matrix, sorted
   double *X0, *X1, *G, *B, *SX, *E, *SXs;
-  float* part;          // 4 x gridDim.x: partial norms, largest correction, partial norms of the block
+  double* part;         // 4 x gridDim.x: partial sums of squares of X^T X - I, of the off-diagonal X^T S X, of
+                        // its pairs with the block, of S
+  float* big;           // gridDim.x: largest correction
   double tau_next;      // threshold of the next level (0: none)
   PsdState* st;
 };
@@ -595,14 +587,21 @@ __device__ double pr_tile(const double* A, int lda, bool acol, int i0, int I, co
   return s;
 }
 
-__device__ __forceinline__ float pr_block_sum(float v, float* redf) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+// Sums over the CTA of v0 and v1, held by the lanes l = tid % 4 = 0, to out0[0] and out1[0]; red: 16 doubles, not
+// used again before the next CTA barrier.  Both go through the same additions, on lanes l = 0 and 1.
+__device__ __forceinline__ void pr_block_pair(double v0, double v1, double* red, double* out0, double* out1) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = lane & 3;
+  const double up = __shfl_up_sync(0xffffffffu, v1, 1);
+  double v = l == 0 ? v0 : l == 1 ? up : 0.0;
+  for (int o = 16; o > 2; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane < 2) red[2 * w + lane] = v;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float s = 0.f;
-  for (int w = 0; w < PR_THREADS / 32; ++w) s += redf[w];
-  return s;
+  if (w == 0) {
+    v = lane < 2 * (PR_THREADS / 32) ? red[lane] : 0.0;
+    for (int o = PR_THREADS / 32; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) *out0 = v;
+    if (lane == 1 && out1) *out1 = v;
+  }
 }
 
 // Order-preserving integer key of a double, NaN below everything.
@@ -614,14 +613,14 @@ __device__ __forceinline__ long long pr_key(double v) {
 
 // Symmetric product P = U^T W (both K x n, row-major; the upper tiles, mirrored) and, when T is
 // given, T = L R with L (M x n, row-major) and R (n x n): the tiles of both dealt to the CTAs.
-// Sum of squares of (delta_ij - P_ij) (of_identity) or of the off-diagonal P_ij, all and (tail) those
-// with a column at t0 or beyond.
-__device__ float pr_products(const PsdGrid& g, int n, const double* U, const double* W, int K, double* P,
-                             bool of_identity, const double* L, const double* R, int M, double* T, int t0, float& tail,
+// Sum of squares of (delta_ij - P_ij) (of_identity) or of the off-diagonal P_ij and, of the latter, (tail) of those
+// with a column at t0 or beyond; in FP64, as couplings of the deep levels square to below FP32's range.  On
+// the lanes tid % 4 = 0.
+__device__ double pr_products(const PsdGrid& g, int n, const double* U, const double* W, int K, double* P,
+                             bool of_identity, const double* L, const double* R, int M, double* T, int t0, double& tail,
                              double* sA, double* sB) {
   const int nt = (n + PR_T - 1) / PR_T, sym = nt * (nt + 1) / 2, mt = T ? (M + PR_T - 1) / PR_T : 0;
-  float nrm = 0.f;
-  tail = 0.f;
+  double diag = 0.0, off = 0.0, offt = 0.0;
   const int tid = threadIdx.x, l = tid & 3, oi = (tid >> 2) >> 3, oj = (tid >> 2) & 7;
   for (int t = g.b; t < sym + mt * nt; t += g.G) {
     if (t < sym) {
@@ -632,10 +631,12 @@ __device__ float pr_products(const PsdGrid& g, int n, const double* U, const dou
       if (l == 0 && i < n && j < n && i <= j) {
         P[size_t(i) * n + j] = s;
         if (i != j) P[size_t(j) * n + i] = s;
-        const float v = of_identity ? float((i == j ? 1.0 : 0.0) - s) : (i == j ? 0.f : float(s));
-        const float q = (i == j ? 1.f : 2.f) * v * v;
-        nrm += q;
-        if (j >= t0) tail += q;
+        if (i != j) {
+          off = fma(s, s, off);
+          if (t0 > 0 && j >= t0) offt = fma(s, s, offt);
+        } else if (of_identity) {
+          diag = fma(1.0 - s, 1.0 - s, diag);
+        }
       }
     } else {
       const int q = t - sym, a = q / nt, b = q % nt, i = a * PR_T + oi, j = b * PR_T + oj;
@@ -643,7 +644,8 @@ __device__ float pr_products(const PsdGrid& g, int n, const double* U, const dou
       if (l == 0 && i < M && j < n) T[size_t(i) * n + j] = s;
     }
   }
-  return nrm;
+  tail = 2.0 * (t0 > 0 ? offt : off);
+  return fma(2.0, off, diag);
 }
 
 // Xo[:, col(j)] = X + X E (mode 0), X (3 I - E) / 2 (mode 1), X E (mode 2); rank: column map or null.
@@ -673,16 +675,13 @@ __device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
   double* sl = sB + PR_T * Kmax;            // n eigenvalues
   int* rank = reinterpret_cast<int*>(sl + n);
   __shared__ float redf[PR_THREADS / 32];
-  __shared__ float delta_s, delta_t;
+  __shared__ double red[2 * (PR_THREADS / 32)], norms[4], delta_s, delta_t;
   __shared__ float tail_s;
   __shared__ float slf[PS_MAX_N];
   __shared__ int flag;
   unsigned int target = 0;
   const int t0 = a.level > 0 ? st->t0 : 0;
-  const float an = float(st->anorm);
-  // the largest eigenvalue of the level's block (sorted by the level before)
-  const float an_tail = a.level > 0 && t0 < n ? float(a.lam[t0]) : an;
-  float unused;
+  double unused;
   double* X = a.X0;
   double* Xn = a.X1;
   bool ok = true;
@@ -706,27 +705,28 @@ __device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
     __syncthreads();
   };
   auto xtsx1 = [&]() {   // G = X^T X and B = F X or S X
-    float tl;
-    const float v = pr_products(g, n, X, X, n, a.G, true, a.F ? a.F : a.S, X, a.F ? a.m : n, a.B, t0, tl, sA, sB);
-    const float s = pr_block_sum(v, redf);
-    if (tid == 0) a.part[g.b] = s;
+    double tl;
+    const double v = pr_products(g, n, X, X, n, a.G, true, a.F ? a.F : a.S, X, a.F ? a.m : n, a.B, n, tl, sA, sB);
+    pr_block_pair(v, 0.0, red, a.part + g.b, nullptr);
   };
   auto xtsx2 = [&]() {                  // SX = B^T B or X^T B
-    float tl;
-    const float v = pr_products(g, n, a.F ? a.B : X, a.B, a.F ? a.m : n, a.SX, false, nullptr, nullptr, 0, nullptr, t0, tl,
-                                sA, sB);
-    const float s = pr_block_sum(v, redf);
-    const float st_ = pr_block_sum(tl, redf);
-    if (tid == 0) {
-      a.part[G + g.b] = s;
-      a.part[3 * G + g.b] = st_;
-    }
+    double tl;
+    const double v = pr_products(g, n, a.F ? a.B : X, a.B, a.F ? a.m : n, a.SX, false, nullptr, nullptr, 0, nullptr, t0, tl,
+                                 sA, sB);
+    pr_block_pair(v, tl, red, a.part + G + g.b, a.part + 2 * G + g.b);
   };
   do {
     // ---- the level's start: X = Y, or X = V diag(I, Y)
     const int nt0 = n - t0;
     if (a.level == 0) {
-      for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) X[e] = a.Y[e];
+      double f = 0.0;
+      for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS) {
+        X[e] = a.Y[e];
+        f = fma(a.S[e], a.S[e], f);
+      }
+      f += __shfl_xor_sync(0xffffffffu, f, 1);
+      f += __shfl_xor_sync(0xffffffffu, f, 2);
+      pr_block_pair(f, 0.0, red, a.part + 3 * G + g.b, nullptr);
     } else {
       for (int e = g.b * PR_THREADS + tid; e < n * t0; e += G * PR_THREADS) {
         const int i = e / t0, j = e % t0;
@@ -754,28 +754,29 @@ __device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
       if (!(ok = pr_sync(st, g, target, &flag))) break;
       xtsx2();
       if (!(ok = pr_sync(st, g, target, &flag))) break;
-      lambda();
-      if (tid < 32) {
-        float ro = 0.f, so = 0.f, tl = 0.f;
-        for (int i = tid; i < G; i += 32) {
-          ro += __ldcg(a.part + i);
-          so += __ldcg(a.part + G + i);
-          tl += __ldcg(a.part + 3 * G + i);
+      // the resolution of the eigenvalue estimates, on the warps that lambda() leaves idle (n <= 128): one a
+      // sum, then 2 (||off-diagonal|| + ||S|| ||X^T X - I||) and the same for the level's block
+      if (tid >= 128) {
+        const int q = (tid >> 5) - 4, lane = tid & 31;
+        if (q < 3 || (a.level == 0 && it == 0)) {
+          double v = 0.0;
+          for (int i = lane; i < G; i += 32) v += __ldcg(a.part + q * G + i);
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) norms[q] = sqrt(v);
+        } else if (it == 0 && lane == 0) {
+          norms[3] = __ldcg(&st->anorm);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-          ro += __shfl_xor_sync(0xffffffffu, ro, o);
-          so += __shfl_xor_sync(0xffffffffu, so, o);
-          tl += __shfl_xor_sync(0xffffffffu, tl, o);
-        }
-        if (tid == 0) {
-          delta_s = 2.f * (sqrtf(so) + an * sqrtf(ro));
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (tid == 128) {
+          delta_s = 2.0 * fma(norms[3], norms[0], norms[1]);
           // pairs with the level's block: with a factor their entries carry errors on their own
-          // scale, so the couplings among the columns above it do not hold them back
-          delta_t = a.F ? 2.f * (sqrtf(tl) + an_tail * sqrtf(ro)) : delta_s;
+          // scale, so the couplings among the columns above it do not hold them back; the block's
+          // largest eigenvalue comes from the level before
+          delta_t = a.F ? 2.0 * fma(a.level > 0 && t0 < n ? __ldcg(a.lam + t0) : norms[3], norms[0], norms[2]) : delta_s;
         }
       }
-      __syncthreads();
-      const double delta_all = double(delta_s), delta_tail = double(delta_t);
+      lambda();
+      const double delta_all = delta_s, delta_tail = delta_t;
       // the next level's threshold, if its tail starts among the kept ones (it is then taken)
       // (comparisons in FP32: an FP64 one takes a slot of the FP64 pipe)
       const float fi_ = tid < n ? slf[tid] : 0.f;
@@ -812,14 +813,14 @@ __device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
       __syncthreads();
       if (tid == 0) {
         for (int w = 1; w < PR_THREADS / 32; ++w) big = fmaxf(big, redf[w]);
-        a.part[2 * G + g.b] = big;
+        a.big[g.b] = big;
       }
       if (!(ok = pr_sync(st, g, target, &flag))) break;
       pr_update(g, n, X, a.E, Xn, 0, nullptr, sA, sB);
       swap();
       // the same decision in every CTA: the largest correction of this iteration
       float mb = 0.f;
-      for (int i = tid & 31; i < G; i += 32) mb = fmaxf(mb, __ldcg(a.part + 2 * G + i));
+      for (int i = tid & 31; i < G; i += 32) mb = fmaxf(mb, __ldcg(a.big + i));
       for (int o = 16; o > 0; o >>= 1) mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
       if (!(ok = pr_sync(st, g, target, &flag))) break;
       // corrections shrink quadratically where the gaps resolve a pair, by a constant factor while a
@@ -845,6 +846,7 @@ __device__ __forceinline__ bool psd_level(const PsdArgs& a, const PsdGrid& g) {
       for (int e = g.b * PR_THREADS + tid; e < n * n; e += G * PR_THREADS)
         a.SXs[size_t(rank[e / n]) * n + rank[e % n]] = __ldcg(a.SX + e);
     if (g.b == 0) {
+      if (a.level == 0 && tid == 0) st->anorm = norms[3];
       for (int i = tid; i < n; i += PR_THREADS) {
         a.lam[rank[i]] = sl[i];
         a.w[rank[i]] = ldexp(sl[i], st->e);
@@ -927,7 +929,7 @@ void eigh_psd(Ctx& c, int n, const double* S, double* w, double* V, int keep, co
   const int tiles = nt * (nt + 1) / 2 + nt * (F ? (m + PR_T - 1) / PR_T : nt);
   const int G = std::max(1, std::min(tiles, &c == c.root ? c.num_sms : std::max(1, c.num_sms / 2)));
   DBuf Ssc(&c, nn), Y(&c, nn), X0(&c, nn), X1(&c, nn), Gm(&c, nn), B(&c, size_t(std::max(m, n)) * n), SX(&c, nn),
-      E(&c, nn), SXs(&c, nn), lam(&c, size_t(n)), part(&c, size_t(2) * G), stb(&c, (sizeof(PsdState) + 7) / 8),
+      E(&c, nn), SXs(&c, nn), lam(&c, size_t(n)), part(&c, size_t(5) * G), stb(&c, (sizeof(PsdState) + 7) / 8),
       Fsc(&c, F ? size_t(m) * n : 1);
   PsdState* st = reinterpret_cast<PsdState*>(stb.p);
   ProfScope ps(c, KC_EIG);
@@ -944,7 +946,8 @@ void eigh_psd(Ctx& c, int n, const double* S, double* w, double* V, int keep, co
   a.n = n; a.m = F ? m : 0; a.keep = keep;
   a.S = Ssc.p; a.F = F ? Fsc.p : nullptr; a.Y = Y.p; a.V = V; a.w = w; a.lam = lam.p;
   a.X0 = X0.p; a.X1 = X1.p; a.G = Gm.p; a.B = B.p; a.SX = SX.p; a.E = E.p; a.SXs = SXs.p;
-  a.part = reinterpret_cast<float*>(part.p);
+  a.part = part.p;
+  a.big = reinterpret_cast<float*>(part.p + 4 * size_t(G));
   a.st = st;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(G));
