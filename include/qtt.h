@@ -146,7 +146,7 @@ typedef struct {
 #define QTT_SOLVE_STALLED 1
 #define QTT_SOLVE_MAX_SWEEPS 2
 #define QTT_SOLVE_NONFINITE 3     /* the residual became NaN or Inf */
-#define QTT_SOLVE_TIMEOUT 4       /* a bounded grid barrier of a local CG solve ran out */
+#define QTT_SOLVE_TIMEOUT 4       /* a bounded wait (a barrier of a local CG solve; a QR) ran out */
 
 typedef struct {
   int sweeps;              /* full sweeps done */
@@ -187,14 +187,18 @@ int qtt_ctx_profile(qtt_ctx* ctx, int on, double* ms_out, double* flops_out, int
  * with momentum, unused, Poisson, projection -- row 5 = outside any phase; column k = kernel
  * class k), and launches_out[6] (kernel launches enqueued in each row).  Either may be NULL. */
 int qtt_ctx_profile_phases(qtt_ctx* ctx, double* ms_out, int64_t* launches_out);
-/* Limit (seconds, > 0) of every bounded device wait of this context: the barriers of the one-kernel
- * CG solves (default 2 s).  A wait that runs out makes its kernel leave at once;
+/* Limit (seconds, > 0) of the barriers of this context's kernels (default 2 s): those of the one-kernel CG
+ * solves, overlaps and eigenproblems.  In a CG solve a wait that runs out makes its kernel leave at once;
  * the solve then ends with QTT_SOLVE_TIMEOUT and the call returns QTT_ERR_TIMEOUT, with the
  * context still usable.  Takes effect for work enqueued afterwards (a captured step keeps the
  * limit it was captured with: set it before the first fractional_step or after
  * qtt_case_use_graph).  Tests shorten it to exercise the timeout path without any fault.
  * The values of overlaps and of the roundings' eigenproblems do not depend on the limit: where a wait
- * of the one-kernel overlap or of the eigensolver's grid runs out, the work is done again without waits. */
+ * of the one-kernel overlap or of the eigensolver's grid runs out, the work is done again without waits.
+ * The waits of the cluster QR, between CTAs that are resident together, do not follow the limit: they end
+ * after 2 s, and the call, or for a call that reads nothing back the next one of the context that does
+ * (qtt_ctx_sync among them), returns QTT_ERR_TIMEOUT, once; what was computed since the last such
+ * call is not valid then. */
 int qtt_ctx_set_wait_limit(qtt_ctx* ctx, double seconds);
 /* How ALS local systems are solved (Sec. II.A.4).  Mode 2 runs each local CG solve as one
  * cooperative kernel on the FP64 pipe (one CTA per SM, grid barriers between its stages) where
@@ -298,6 +302,9 @@ int qtt_sym_eig(qtt_ctx* ctx, int n, const double* S, double* w, double* V);
  * (QTT_ERR_UNSUPPORTED if the shape does not allow it).  Host buffers; R may be NULL;
  * synchronous. */
 int qtt_qr(qtt_ctx* ctx, int m, int n, int trans, const double* A, double* Q, double* R, int path);
+/* Self-check of the report of an expired wait (qtt_ctx_set_wait_limit): enqueues one cluster QR of an
+ * m x n matrix whose waits are limited to `seconds`, and reads nothing back. */
+int qtt_check_qr_wait(qtt_ctx* ctx, int m, int n, double seconds);
 /* C = A B for row-major host matrices A (m x k), B (k x n), C (m x n); synchronous.  The product
  * behind every core contraction of the sweeps (Sec. II.A).  path 0 uses the context's mode (see
  * qtt_ctx_set_gemm_mode), 1 forces the FP64 pipe, 2 and 3 force the tensor-core product: every row
@@ -343,7 +350,7 @@ int mps_dot(qtt_ctx* ctx, const qtt_mps* a, const qtt_mps* b, double* out_host);
  * qtt_solve_opts: x_inout is the warm start and receives the solution (its bond profile is
  * kept).  Blocks the host until the solve has finished.  Returns QTT_OK when the residual met
  * opts->rel_tol, QTT_ERR_NOT_CONVERGED when the solve stalled or ran out of sweeps (x_inout then
- * holds the last iterate), QTT_ERR_TIMEOUT when a grid barrier ran out, QTT_ERR_NONFINITE when
+ * holds the last iterate), QTT_ERR_TIMEOUT when a bounded wait ran out, QTT_ERR_NONFINITE when
  * the residual became NaN or Inf; info (may be NULL) is filled in every one of these cases.
  * n <= 30 (the residual is evaluated on 2^n entries). */
 int poisson_solve(qtt_ctx* ctx, const qtt_mpo* A, const qtt_mps* b, qtt_mps* x_inout,
@@ -392,7 +399,7 @@ int qtt_case_get_operator(qtt_case* c, int which, qtt_mpo** out);
 int qtt_case_get_vector(qtt_case* c, int which, qtt_mps** out);
 /* Advance nsteps fractional steps (Sec. III.C) and block the host until they have finished.
  * per_step (may be NULL) receives nsteps records.  Forces are evaluated when with_forces != 0
- * and per_step is given.  Returns QTT_ERR_TIMEOUT if a local CG barrier ran out, QTT_ERR_NONFINITE
+ * and per_step is given.  Returns QTT_ERR_TIMEOUT if a bounded wait ran out, QTT_ERR_NONFINITE
  * if a residual or a new velocity norm was NaN or Inf, QTT_ERR_NOT_CONVERGED if a solve used all
  * of its sweeps without meeting its tolerance (a stall at the bond's floor is not an error),
  * checked over all steps whether or not per_step is given. */

@@ -345,6 +345,7 @@ qtt_mps* round_svd(Ctx& c, const qtt_mps* x_in, int chi, double eps) {
     std::vector<double> sig(nn);
     QTT_CUDA(cudaMemcpyAsync(sig.data(), S.p, nn * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
     QTT_CUDA(cudaStreamSynchronize(c.stream));
+    check_waits(c);
     int nz = 0;
     for (double s : sig)
       if (s > 0.0) ++nz;
@@ -401,6 +402,7 @@ static std::vector<double> host_copy(Ctx& c, const double* p, int n) {
   std::vector<double> h(n);
   QTT_CUDA(cudaMemcpyAsync(h.data(), p, n * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   QTT_CUDA(cudaStreamSynchronize(c.stream));
+  check_waits(c);
   return h;
 }
 
@@ -1192,6 +1194,7 @@ double dot_host(Ctx& c, const qtt_mps* a, const qtt_mps* b) {
     QTT_CUDA(cudaMemcpyAsync(v, out.p, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
     QTT_CUDA(cudaStreamSynchronize(c.stream));
   }
+  check_waits(c);
   return v[0];
 }
 

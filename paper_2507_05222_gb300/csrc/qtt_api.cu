@@ -17,6 +17,18 @@ namespace qtt {
 static thread_local std::string g_last_error;
 void set_last_error(const std::string& msg) { g_last_error = msg; }
 
+bool waits_expired(Ctx& c) {
+  volatile unsigned int* w = c.root->wait_word;
+  if (!w || *w == 0u) return false;
+  *w = 0u;
+  return true;
+}
+
+static const char* const kWaitText = "a wait between the CTAs of a QR timed out: results since the last read-back are not valid";
+void check_waits(Ctx& c) {
+  if (waits_expired(c)) throw Error(QTT_ERR_TIMEOUT, kWaitText);
+}
+
 }  // namespace qtt
 
 using namespace qtt;
@@ -81,7 +93,7 @@ int solve_status_code(int status, bool floor_ok = false) {
 
 std::string solve_status_text(const AlsCtl& h) {
   static const char* names[] = {"converged", "stalled above the tolerance", "out of sweeps", "non-finite residual",
-                                "a CG grid barrier timed out"};
+                                "a bounded wait timed out"};
   const char* s = (h.status >= 0 && h.status <= 4) ? names[h.status] : "did not finish";
   return std::string(s) + " after " + std::to_string(h.sweeps) + " sweeps, relative residual " +
          std::to_string(h.res);
@@ -180,6 +192,9 @@ int qtt_ctx_create(qtt_ctx** out, int device, void* cuda_stream, qtt_alloc_fn al
   c->alloc_fn = alloc;
   c->free_fn = free_fn;
   c->alloc_user = user;
+  QTT_CUDA(cudaHostAlloc(&c->wait_word, sizeof(unsigned int), cudaHostAllocMapped));
+  *c->wait_word = 0u;
+  QTT_CUDA(cudaHostGetDevicePointer(&c->wait_word_dev, c->wait_word, 0));
   init_tile_counters(*c);
   *out = reinterpret_cast<qtt_ctx*>(c.release());
   API_END
@@ -200,6 +215,7 @@ void qtt_ctx_destroy(qtt_ctx* ctx) {
   free_autotuner(*c);
   if (c->prof.dev_flops) cudaFree(c->prof.dev_flops);
   if (c->side) cudaStreamDestroy(c->side);
+  if (c->wait_word) cudaFreeHost(c->wait_word);
   delete c->pool;
   delete c;
 }
@@ -208,6 +224,7 @@ int qtt_ctx_sync(qtt_ctx* ctx) {
   API_BEGIN
   QTT_CHECK_ARG(ctx, "ctx is null");
   QTT_CUDA(cudaStreamSynchronize(reinterpret_cast<Ctx*>(ctx)->stream));
+  check_waits(*reinterpret_cast<Ctx*>(ctx));
   API_END
 }
 
@@ -348,7 +365,10 @@ int qtt_mps_get_cores(const qtt_mps* x, double* dst, int kind) {
     QTT_CUDA(cudaMemcpyAsync(dst + o, x->core(i), sz * sizeof(double), k, c.stream));
     o += sz;
   }
-  if (kind == QTT_HOST) QTT_CUDA(cudaStreamSynchronize(c.stream));
+  if (kind == QTT_HOST) {
+    QTT_CUDA(cudaStreamSynchronize(c.stream));
+    check_waits(c);
+  }
   API_END
 }
 
@@ -429,9 +449,9 @@ int qtt_encode(qtt_ctx* ctx, const double* dense, int kind, int n, int d, qtt_tr
   DBuf buf(&c, size_t(N));
   QTT_CUDA(cudaMemcpyAsync(buf.p, dense, N * sizeof(double), kind_in(kind), c.stream));
   DiscScope disc(c, info != nullptr);
-  qtt_mps* y = encode_dense(c, buf.p, n, d, tr.chi_max, tr.rel_tol);
-  fill_info(c, y, info, &disc);
-  *out = y;
+  std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> y(encode_dense(c, buf.p, n, d, tr.chi_max, tr.rel_tol), free_mps);
+  fill_info(c, y.get(), info, &disc);
+  *out = y.release();
   API_END
 }
 
@@ -450,6 +470,7 @@ int qtt_decode(qtt_ctx* ctx, const qtt_mps* x, double* dense, int kind) {
     decode_mid(c, x, buf.p);
     QTT_CUDA(cudaMemcpyAsync(dense, buf.p, N * sizeof(double), kind_out(kind), c.stream));
     QTT_CUDA(cudaStreamSynchronize(c.stream));
+    check_waits(c);
   }
   API_END
 }
@@ -480,9 +501,9 @@ int qtt_round(qtt_ctx* ctx, const qtt_mps* x, qtt_trunc tr, qtt_mps** out, qtt_r
   Ctx& c = *reinterpret_cast<Ctx*>(ctx);
   DigitsScope prec(c, prec_digits(tr.prec));
   DiscScope disc(c, info != nullptr);
-  qtt_mps* y = round_any(c, x, tr.chi_max, tr.rel_tol);
-  fill_info(c, y, info, &disc);
-  *out = y;
+  std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> y(round_any(c, x, tr.chi_max, tr.rel_tol), free_mps);
+  fill_info(c, y.get(), info, &disc);
+  *out = y.release();
   API_END
 }
 
@@ -499,9 +520,9 @@ int mps_axpby_round(qtt_ctx* ctx, double alpha, const qtt_mps* x, double beta, c
   DigitsScope prec(c, prec_digits(tr.prec));
   std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> s(direct_sum(c, alpha, x, beta, y), free_mps);
   DiscScope disc(c, info != nullptr);
-  qtt_mps* z = round_any(c, s.get(), tr.chi_max, tr.rel_tol);
-  fill_info(c, z, info, &disc);
-  *out = z;
+  std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> z(round_any(c, s.get(), tr.chi_max, tr.rel_tol), free_mps);
+  fill_info(c, z.get(), info, &disc);
+  *out = z.release();
   API_END
 }
 
@@ -514,18 +535,18 @@ int mpo_apply_round(qtt_ctx* ctx, const qtt_mpo* M, const qtt_mps* x, qtt_trunc 
   check_trunc(tr);
   Ctx& c = *reinterpret_cast<Ctx*>(ctx);
   DigitsScope prec(c, prec_digits(tr.prec));
-  qtt_mps* y;
+  std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> y(nullptr, free_mps);
   DiscScope disc(c, info != nullptr);
   if (tr.rel_tol > 0.0) {
     std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> e(mpo_mps_exact(c, M, x), free_mps);
-    y = round_any(c, e.get(), tr.chi_max, tr.rel_tol);
+    y.reset(round_any(c, e.get(), tr.chi_max, tr.rel_tol));
   } else if (tr.apply == QTT_APPLY_SKETCH) {
-    y = apply_round_sketch(c, M, x, tr.chi_max, 0.0);
+    y.reset(apply_round_sketch(c, M, x, tr.chi_max, 0.0));
   } else {
-    y = apply_round_gram(c, M, x, tr.chi_max, 0.0);
+    y.reset(apply_round_gram(c, M, x, tr.chi_max, 0.0));
   }
-  fill_info(c, y, info, &disc);
-  *out = y;
+  fill_info(c, y.get(), info, &disc);
+  *out = y.release();
   API_END
 }
 
@@ -586,6 +607,18 @@ int qtt_qr(qtt_ctx* ctx, int m, int n, int trans, const double* A, double* Q, do
   QTT_CUDA(cudaMemcpyAsync(Q, dQ.p, size_t(m) * kk * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   if (R) QTT_CUDA(cudaMemcpyAsync(R, dR.p, size_t(kk) * n * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   QTT_CUDA(cudaStreamSynchronize(c.stream));
+  check_waits(c);
+  API_END
+}
+
+int qtt_check_qr_wait(qtt_ctx* ctx, int m, int n, double seconds) {
+  API_BEGIN
+  QTT_CHECK_ARG(ctx && m >= 1 && n >= 1 && int64_t(m) * n <= (int64_t(1) << 22), "check_qr_wait: m, n >= 1 and m n <= 2^22");
+  QTT_CHECK_ARG(seconds > 0.0 && seconds <= 3600.0, "check_qr_wait: seconds in (0, 3600]");
+  Ctx& c = *reinterpret_cast<Ctx*>(ctx);
+  DBuf A(&c, size_t(m) * n);
+  fill(c, A.p, int64_t(m) * n, 1.0);
+  qr(c, 1, m, n, 0, A.p, 0, A.p, 0, nullptr, 0, 2, static_cast<unsigned long long>(std::max(1.0, seconds * 1e9)));
   API_END
 }
 
@@ -707,6 +740,7 @@ int poisson_solve(qtt_ctx* ctx, const qtt_mpo* A, const qtt_mps* b, qtt_mps* x_i
   AlsCtl h;
   QTT_CUDA(cudaMemcpyAsync(&h, cp, sizeof(AlsCtl), cudaMemcpyDeviceToHost, c.stream));
   QTT_CUDA(cudaStreamSynchronize(c.stream));
+  if (waits_expired(c)) h.status = QTT_SOLVE_TIMEOUT;
   if (info) fill_solve_info(h, info);
   const int rc = solve_status_code(h.status);
   if (rc != QTT_OK) {
@@ -887,7 +921,11 @@ int fractional_step(qtt_ctx* ctx, qtt_case* h, int nsteps, int with_forces, qtt_
   QTT_CUDA(cudaMemcpyAsync(hrec.data(), rec.p, hrec.size() * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   QTT_CUDA(cudaStreamSynchronize(c.stream));
   std::string msg;
-  const int rc = read_step_records(c, cs, hrec.data(), nsteps, forces, per_step, "fractional_step", msg);
+  int rc = read_step_records(c, cs, hrec.data(), nsteps, forces, per_step, "fractional_step", msg);
+  if (waits_expired(c) && rc != QTT_ERR_TIMEOUT) {
+    rc = QTT_ERR_TIMEOUT;
+    msg = std::string("fractional_step: ") + kWaitText;
+  }
   if (rc != QTT_OK) {
     set_last_error(msg);
     return rc;
@@ -926,11 +964,16 @@ int fractional_step_batch(qtt_ctx* ctx, int ncases, qtt_case* const* cases, int 
   QTT_CUDA(cudaStreamSynchronize(c.stream));
   int rc = QTT_OK;
   std::string first;
+  const bool expired = waits_expired(c);   // which case's QR is not known: all of them are in doubt
   for (int i = 0; i < ncases; ++i) {
     std::string msg;
     const std::string who = "fractional_step_batch: case " + std::to_string(i);
-    const int e = read_step_records(c, *cs[i], hrec.data() + int64_t(i) * nsteps * kStepRecDoubles, nsteps, forces,
-                                    per_step ? per_step + int64_t(i) * nsteps : nullptr, who.c_str(), msg);
+    int e = read_step_records(c, *cs[i], hrec.data() + int64_t(i) * nsteps * kStepRecDoubles, nsteps, forces,
+                              per_step ? per_step + int64_t(i) * nsteps : nullptr, who.c_str(), msg);
+    if (expired && e != QTT_ERR_TIMEOUT) {
+      e = QTT_ERR_TIMEOUT;
+      msg = who + ": " + kWaitText;
+    }
     if (status) status[i] = e;
     if (more_severe(rc, e) != rc) {
       rc = e;
@@ -1140,6 +1183,7 @@ int qtt_case_forces(qtt_ctx* ctx, qtt_case* h, double* cd, double* cl) {
   double hv[2];
   QTT_CUDA(cudaMemcpyAsync(hv, o.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   QTT_CUDA(cudaStreamSynchronize(c.stream));
+  check_waits(c);
   *cd = hv[0];
   *cl = hv[1];
   API_END

@@ -176,8 +176,12 @@ struct Ctx {
   cudaStream_t side = nullptr;
   // When non-null, every TT-SVD cut of a rounding adds its discarded sigma^2 here (device).
   double* disc_acc = nullptr;
-  // Limit of every bounded device wait (grid barriers of the cooperative CG), read from root.
+  // Limit of the bounded device waits (qtt_ctx_set_wait_limit), read from root.
   unsigned long long wait_ns = 2000000000ull;
+  // Set by a kernel whose bounded wait ran out and whose results are therefore not valid (the cluster QR):
+  // one word of host memory that the device writes, read after a synchronisation; root context.
+  unsigned int* wait_word = nullptr;
+  unsigned int* wait_word_dev = nullptr;
   Profiler prof;
   // GEMM autotuner (root context): when autotune is on, a GEMM shape met for the first time is
   // timed under every candidate engine on tune_stream and the fastest is kept in tuned; shapes
@@ -213,6 +217,10 @@ void init_tile_counters(Ctx& c);   // allocate and zero c.tile_ctr (outside stre
 void free_tile_counters(Ctx& c);
 
 void after_launch(Ctx& c, const char* what);
+// After a synchronisation: whether a wait of the cluster QR ran out since the last question, and the same
+// as an error (QTT_ERR_TIMEOUT).  Every call that reads results back asks.
+bool waits_expired(Ctx& c);
+void check_waits(Ctx& c);
 
 Ctx& worker(Ctx& c, int i);     // i-th worker of c (created on first use)
 void fork(Ctx& c, int n);       // workers 0..n-1 wait for the work enqueued on c so far
@@ -318,8 +326,11 @@ void dot(Ctx& c, int64_t n, const double* x, const double* y, double* out_dev);
 // correctly rounded 1/x and 1/sqrt(x) over x_dev[0..n): err_dev[0], err_dev[1].
 void check_recip(Ctx& c, int n, const double* x_dev, double* err_dev);
 // path: 0 = cluster QR when the shape allows it, else one CTA; 1 = one CTA; 2 = cluster only.
+// wait_ns bounds the cluster kernel's waits.  They do not follow qtt_ctx_set_wait_limit: that limit is for solves, and
+// a low one must not end the roundings.
+constexpr unsigned long long kQrWaitNs = 2000000000ull;
 void qr(Ctx& c, int count, int m, int n, int trans, const double* A, int64_t in_stride, double* Q, int64_t q_stride,
-        double* R, int64_t r_stride, int path = 0);
+        double* R, int64_t r_stride, int path = 0, unsigned long long wait_ns = kQrWaitNs);
 // Whether qr() supports an m x n matrix (cluster kernel or one CTA).
 bool qr_fits(int m, int n);
 // Accurate (one-sided Jacobi, FP64) SVD of a small m x n matrix, m >= n: U (m x n), s, V (n x n).

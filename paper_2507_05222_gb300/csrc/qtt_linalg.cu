@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(256) k_qr(int m, int n, int trans, const doubl
 //     R phase of the later ones; the last cs / 4 panels, whose Q would be left over at the end, are
 //     split into four groups of columns, for their owner and three CTAs that are done by then.
 // Each barrier is used once and only later CTAs wait, on earlier ones, so the waits end; they are
-// bounded all the same (a wait that runs out gives NaN).
+// bounded all the same (one that runs out gives NaN and sets *expired, which the host turns into an error).
 // Columns are scaled by powers of two to a largest entry in [1, 2) (R's columns scaled back: exact),
 // so that the squares and products above neither overflow nor underflow.
 // What bounds it: the serial chain of FP64 instructions.  Each takes its sub-partition 64 clocks, dependent or
@@ -278,20 +278,34 @@ __device__ __forceinline__ void qrc_signal(const uint64_t* bar, int rank) {
       "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(qrc_smem_addr(bar)), "r"(rank)
       : "memory");
 }
-// Wait for the one arrival on an own barrier; false after some 4 million tries.
-__device__ __forceinline__ bool qrc_wait(const uint64_t* bar) {
-  for (int k = 0; k < (1 << 22); ++k) {
+// Wait for the one arrival on an own barrier, at most limit_ns by the global timer.  (A try may suspend the
+// thread for a time that the hardware chooses; limits below 0.1 ms, in tests of the expiry, only test.)
+__device__ __forceinline__ bool qrc_wait(const uint64_t* bar, unsigned long long limit_ns) {
+  unsigned long long t0 = 0;
+  while (true) {
     int done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
-        "selp.s32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(qrc_smem_addr(bar))
-        : "memory");
+    if (limit_ns < 100000ull)
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t"
+          "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+          "selp.s32 %0, 1, 0, p;\n\t}"
+          : "=r"(done)
+          : "r"(qrc_smem_addr(bar))
+          : "memory");
+    else
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t"
+          "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+          "selp.s32 %0, 1, 0, p;\n\t}"
+          : "=r"(done)
+          : "r"(qrc_smem_addr(bar))
+          : "memory");
     if (done) return true;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (t0 == 0) t0 = t;
+    else if (t - t0 > limit_ns) return false;
   }
-  return false;
 }
 
 // 2^-e of a column whose largest entry lies in [2^e, 2^(e+1)) from the largest high word without its
@@ -414,7 +428,8 @@ __device__ __forceinline__ void qrc_apply4(const QrcBlock<RPL>& b, double (&x)[R
 }
 template <int RPL, int WPC>
 __device__ void qrc_q_job(int m, int n, int nb, int trans, int q, int P, int cc0, int gw, const double* Acol, const double* T,
-                          const double* ud, const uint64_t* bar_t, bool bad, double* redall, double* Q) {
+                          const double* ud, const uint64_t* bar_t, bool bad, double* redall, double* Q,
+                          unsigned long long limit_ns, int* bad_out) {
   cgrp::cluster_group cl = cgrp::this_cluster();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / WPC, sub = warp % WPC;
   double* red = redall + 32 * (WPC > 1 ? group : 0);
@@ -424,7 +439,7 @@ __device__ void qrc_q_job(int m, int n, int nb, int trans, int q, int P, int cc0
 #pragma unroll
     for (int t = 0; t < RPL; ++t) x[t] = lane + 32 * (sub + WPC * t) == cc0 + c ? 1.0 : 0.0;
     auto load = [&](QrcBlock<RPL>& b, int p, int l0) {
-      if (p != q) ok = qrc_wait(bar_t + p) && ok;
+      if (p != q) ok = ok && qrc_wait(bar_t + p, limit_ns);
       qrc_load_block<RPL, WPC>(b, cl.map_shared_rank(Acol, p), cl.map_shared_rank(T, p), cl.map_shared_rank(ud, p), m, nb,
                                p * nb, l0, min(nb, n - p * nb), lane, sub);
     };
@@ -459,6 +474,7 @@ __device__ void qrc_q_job(int m, int n, int nb, int trans, int q, int P, int cc0
       }
     }
     ok = __all_sync(0xffffffffu, ok);
+    if (!ok) *bad_out = 1;
 #pragma unroll
     for (int t = 0; t < RPL; ++t) {
       const int i = lane + 32 * (sub + WPC * t);
@@ -473,7 +489,8 @@ __device__ void qrc_q_job(int m, int n, int nb, int trans, int q, int P, int cc0
 
 __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb, int trans, const double* __restrict__ Ain,
                                                            double* Qall, double* __restrict__ Rall, int64_t in_stride,
-                                                           int64_t q_stride, int64_t r_stride) {
+                                                           int64_t q_stride, int64_t r_stride,
+                                                           unsigned long long limit_ns, unsigned int* expired) {
   cgrp::cluster_group cl = cgrp::this_cluster();
   const int cs = int(cl.num_blocks());
   const int q = int(cl.block_rank());
@@ -531,7 +548,7 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
   bool ok = true;
   for (int s = 0; s < c0 && s < n && w > 0; ++s) {
     const int p = s / nb, l = s - p * nb;
-    ok = qrc_wait(bar_col + s) && ok;
+    ok = ok && qrc_wait(bar_col + s, limit_ns);   // after a wait that ran out there are no more
     double* u = Vb + size_t(s & 1) * m;
     const double* src = cl.map_shared_rank(Acol, p) + size_t(l) * m;
     for (int i = s + 1 + tid; i < m; i += nt) u[i] = src[i];
@@ -662,7 +679,7 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
     if (gw <= 0) continue;
     const int cc0 = P * nb + g0;
     // one or two columns: four warps each, so that the serial chain of panels is short
-#define QRC_JOB(rpl, wpc) qrc_q_job<rpl, wpc>(m, n, nb, trans, q, P, cc0, gw, Acol, T, ud, bar_t, s_bad != 0, s_red, Q)
+#define QRC_JOB(rpl, wpc) qrc_q_job<rpl, wpc>(m, n, nb, trans, q, P, cc0, gw, Acol, T, ud, bar_t, s_bad != 0, s_red, Q, limit_ns, &s_bad)
     if (m <= 256) {
       if (gw <= 2) {
         if (m <= 128) QRC_JOB(1, 4);
@@ -681,7 +698,7 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
     }
     for (int p = P; p >= 0; --p) {
       const int j0 = p * nb, wp = max(0, min(nb, n - j0)), mr = m - j0;
-      if (p != q) ok = qrc_wait(bar_t + p) && ok;
+      if (p != q) ok = ok && qrc_wait(bar_t + p, limit_ns);
       const double* src = cl.map_shared_rank(Acol, p);
       const double* srcT = cl.map_shared_rank(T, p);
       const double* srcu = cl.map_shared_rank(ud, p);
@@ -703,6 +720,10 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
       else Q[int64_t(i) * n + cc0 + c] = v;         // Q row-major (m x n)
     }
     __syncthreads();
+  }
+  if (tid == 0 && s_bad) {   // set before a CTA barrier that this thread has passed
+    *reinterpret_cast<volatile unsigned int*>(expired) = 1u;
+    __threadfence_system();
   }
   cl.sync();   // no CTA leaves while another may read its panel
 }
@@ -1176,7 +1197,7 @@ bool qr_fits(int m, int n) {
 }
 
 void qr(Ctx& c, int count, int m, int n, int trans, const double* A, int64_t in_stride, double* Q, int64_t q_stride,
-        double* R, int64_t r_stride, int path) {
+        double* R, int64_t r_stride, int path, unsigned long long wait_ns) {
   DigitsScope fp64(c, kDigitsFP64);   // the decompositions and their refinement products stay FP64
   if (count <= 0 || n <= 0 || m <= 0) return;
   init_kernel_attributes();
@@ -1199,7 +1220,8 @@ void qr(Ctx& c, int count, int m, int n, int trans, const double* A, int64_t in_
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    QTT_CUDA(cudaLaunchKernelEx(&cfg, k_qr_cluster, m, n, nb, trans, A, Q, R, in_stride, q_stride, r_stride));
+    QTT_CUDA(cudaLaunchKernelEx(&cfg, k_qr_cluster, m, n, nb, trans, A, Q, R, in_stride, q_stride, r_stride, wait_ns,
+                                c.root->wait_word_dev));
     after_launch(c, "qr_cluster");
     return;
   }

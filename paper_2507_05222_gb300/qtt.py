@@ -107,6 +107,7 @@ _SIGS = {
     "qtt_qr": (I, [P, I, I, I, DP, DP, DP, I]),
     "qtt_ctx_set_cg_mode": (I, [P, I]),
     "qtt_ctx_set_wait_limit": (I, [P, D]),
+    "qtt_check_qr_wait": (I, [P, I, I, D]),
     "qtt_check_recip": (I, [P, I, DP, DP]),
     "qtt_dgemm": (I, [P, I, I, I, DP, DP, DP, I]),
     "qtt_ctx_set_gemm_mode": (I, [P, I]),
@@ -257,7 +258,8 @@ class Context:
                 for i, k in enumerate(self.PROFILE_CLASSES)}
 
     def set_wait_limit(self, seconds: float):
-        """Limit of every bounded device wait (grid barriers of the cooperative CG), default 2 s."""
+        """Limit of the kernels' barriers, default 2 s: a CG solve past it times out, overlaps and roundings
+        are done again without waits (include/qtt.h)."""
         _check(lib().qtt_ctx_set_wait_limit(self.h, float(seconds)))
 
     def set_precision(self, prec: str):
@@ -548,6 +550,11 @@ def qtt_check_recip(ctx: Context, x):
     err = np.zeros(2)
     _check(lib().qtt_check_recip(ctx.h, x.size, _dp(x), _dp(err)))
     return float(err[0]), float(err[1])
+
+
+def qtt_check_qr_wait(ctx: Context, m: int, n: int, seconds: float):
+    """One cluster QR with its waits limited to ``seconds``; an expired one is reported by the next read-back."""
+    _check(lib().qtt_check_qr_wait(ctx.h, int(m), int(n), float(seconds)))
 
 
 def qtt_qr(ctx: Context, A, trans: bool = False, path: int = 0):

@@ -1,10 +1,11 @@
 """The wait limit (qtt_ctx_set_wait_limit) outside the solves.  Overlaps and roundings are completed
 without waits when one runs out, so that their values do not depend on the limit; with a limit of 1 ns
-some wait of every kernel that has grid barriers runs out."""
+some wait of every kernel that has grid barriers runs out.  The waits of the cluster QR have a limit of
+their own, and one that runs out is reported by the next call that reads results back."""
 import numpy as np
 import pytest
 
-from oracle import tt
+from oracle import qtt_ops as Q, step as S, tt
 from paper_2507_05222_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -72,3 +73,52 @@ def test_sketched_product_does_not_depend_on_the_limit(ctx, h, chi, decades):
         ctx.set_wait_limit(limit)
         v = qtt.qtt_decode(ctx, qtt.mpo_apply_round(ctx, gM, gx, chi, apply="sketch")).reshape(N, N)
         assert np.linalg.norm(v - best) <= 1e-11 * np.linalg.norm(best)
+
+
+def readers(qtt, ctx):
+    """Calls that read results back."""
+    ne = 3
+    ops = Q.Ops(ne, ne, 40.0, 100.0, 2e-3, "interleaved")
+    cores = inputs.random_cores(2 * ne, 4, seed=1)
+    g = qtt.MPS.from_cores(ctx, cores)
+    A, b = qtt.MPO.from_cores(ctx, ops.Ap), qtt.MPS.from_cores(ctx, inputs.random_cores(2 * ne, 4, seed=80))
+    def case():
+        u, v = (ops.encode(f, 8) for f in (1.0 + inputs.gaussian_field(ne, ne, 1, 1e-3), inputs.gaussian_field(ne, ne, 2, 1e-3)))
+        p = S.padded([np.zeros((1, 2, 1))] * (2 * ne), 8, inputs.random_cores(2 * ne, 8, 3, scale=1e-8))
+        c = qtt.Case(ctx, ne, ne, 40.0, 100.0, 2e-3, 8, "interleaved")
+        c.set_state(*(qtt.MPS.from_cores(ctx, x) for x in (u, v, p)))
+        return c
+    one, two = case(), case()
+    return {"sync": ctx.sync, "dot": lambda: qtt.mps_dot(ctx, g, g), "decode": lambda: qtt.qtt_decode(ctx, g),
+            "cores": g.cores, "round": lambda: qtt.qtt_round(ctx, g, 4, out_info={}),
+            "threshold": lambda: qtt.qtt_round(ctx, g, 4, rel_tol=1e-3), "qr": lambda: qtt.qtt_qr(ctx, np.eye(64), path=2),
+            "solve": lambda: qtt.poisson_solve(ctx, A, b, qtt.MPS.from_cores(ctx, inputs.random_cores(2 * ne, 8, seed=81)),
+                                               8, 1e-9, 300, 1e-2, 0.1),
+            "step": lambda: one.fractional_step(1), "forces": one.forces,
+            "batch": lambda: qtt.fractional_step_batch(ctx, [one, two], 1)}
+
+
+def test_expired_qr_wait_is_reported_once(ctx):
+    """A cluster QR with a limit of 1 ns gives up; the next call that reads back returns
+    QTT_ERR_TIMEOUT, the one after that works."""
+    from paper_2507_05222_gb300 import qtt
+    calls = readers(qtt, ctx)
+    for f in calls.values():
+        f()
+    for m, n in ((64, 32), (128, 64), (256, 128), (320, 160), (16, 16)):
+        qtt.qtt_check_qr_wait(ctx, m, n, 1e-9)
+        with pytest.raises(qtt.QttError) as e:
+            ctx.sync()
+        assert e.value.code == -5 and "timed out" in str(e.value)
+        qtt.qtt_check_qr_wait(ctx, m, n, 2.0)
+        ctx.sync()
+    for name, f in calls.items():
+        qtt.qtt_check_qr_wait(ctx, 128, 64, 1e-9)
+        with pytest.raises(qtt.QttError) as e:
+            f()
+        assert e.value.code == -5, name
+        f()
+    ctx.set_wait_limit(1e-9)                      # the QR's waits do not follow the limit of the solves
+    A = inputs.rng(3).standard_normal((128, 64))
+    q, r = qtt.qtt_qr(ctx, A, path=2)
+    assert np.linalg.norm(q @ r - A) <= 1e-13 * np.linalg.norm(A)
