@@ -320,9 +320,9 @@ int qtt_dgemm(qtt_ctx* ctx, int m, int n, int k, const double* A, const double* 
  * bit-identical results.
  * Takes effect for work enqueued afterwards (a captured step keeps its kernels). */
 int qtt_ctx_set_gemm_mode(qtt_ctx* ctx, int mode);
-/* Self-check of the QR's Householder scalars: the maximum relative errors of its Newton-Raphson
- * reciprocal (err2[0]) and reciprocal square root (err2[1]) against CUDA's correctly rounded
- * 1/x and 1/sqrt(x) over the n positive host values x.  Synchronous. */
+/* Self-check of the QR's Householder scalars: the maximum relative errors of its reciprocal
+ * (err2[0]) and square root (err2[1]), one third-order step each, against CUDA's correctly rounded
+ * 1/x and sqrt(x) over the n positive host values x.  Synchronous. */
 int qtt_check_recip(qtt_ctx* ctx, int n, const double* x, double* err2);
 /* GEMM autotuner (the contractions that reach the batched GEMM: core products of the
  * environments, the fits and the local solves outside the cooperative CG kernels).  on = 1:

@@ -322,8 +322,8 @@ void dot(Ctx& c, int64_t n, const double* x, const double* y, double* out_dev);
 
 // Householder QR of `count` matrices (strided): A (m x n) = Q (m x kk) R (kk x n), kk = min(m,n).
 // trans = 1: the buffer holds A^T (n x m row-major) and Q^T (kk x m) is written.
-// Max relative errors of the QR's Newton reciprocal / reciprocal square root against CUDA's
-// correctly rounded 1/x and 1/sqrt(x) over x_dev[0..n): err_dev[0], err_dev[1].
+// Max relative errors of the QR's reciprocal / square root against CUDA's
+// correctly rounded 1/x and sqrt(x) over x_dev[0..n): err_dev[0], err_dev[1].
 void check_recip(Ctx& c, int n, const double* x_dev, double* err_dev);
 // path: 0 = cluster QR when the shape allows it, else one CTA; 1 = one CTA; 2 = cluster only.
 // wait_ns bounds the cluster kernel's waits.  They do not follow qtt_ctx_set_wait_limit: that limit is for solves, and

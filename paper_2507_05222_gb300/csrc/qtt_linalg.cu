@@ -173,10 +173,10 @@ __global__ void __launch_bounds__(256) k_qr(int m, int n, int trans, const doubl
 // (nb x nb each) | ud (nb).
 constexpr int QRC_THREADS = 256;
 
-// 1/x and 1/sqrt(x) from the hardware's approximate FP64 reciprocal (square root), ~20 correct bits,
-// by one third-order step each: with e = 1 - x y (or 1 - x y^2), y (1 + e + e^2) and
-// y (1 + e / 2 + 3 e^2 / 8) are good to e^3.  An FP64 division or square root is a sequence of ~10
-// dependent FP64 operations, ~650 cycles on this part; these take 3 x 64 and 4 x 64 cycles.  Results
+// 1/x and sqrt(x), the scalars of a reflector, from the hardware's approximate FP64 reciprocal (square
+// root) y, ~20 correct bits, by one third-order step each: with e = 1 - x y, y (1 + e + e^2), and with n = x y
+// and e = 1 - n y, n (1 + e / 2 + 3 e^2 / 8), are good to e^3.  An FP64 division or square root is a sequence of
+// ~10 dependent FP64 operations, ~650 cycles on this part; these take 3 x 64 and 5 x 64 cycles.  Results
 // are within a few ulp of the correctly rounded ones (checked against CUDA's by qtt_check_recip).
 __device__ __forceinline__ double rcp_nr(double x) {
   double y;
@@ -184,22 +184,22 @@ __device__ __forceinline__ double rcp_nr(double x) {
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double rsqrt_nr(double x) {
+__device__ __forceinline__ double sqrt_nr(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
+  const double n = x * y, e = fma(-n, y, 1.0);
+  return fma(n * e, fma(0.375, e, 0.5), n);
 }
 
 __global__ void k_check_recip(int n, const double* __restrict__ x, double* __restrict__ err) {
-  // err[0] = max relative error of rcp_nr, err[1] of rsqrt_nr, against CUDA's 1/x, 1/sqrt(x)
+  // err[0] = max relative error of rcp_nr, err[1] of sqrt_nr, against CUDA's 1/x, sqrt(x)
   __shared__ double red[2][32];
   double e0 = 0.0, e1 = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const double v = x[i];
-    const double a = 1.0 / v, b = 1.0 / sqrt(v);
+    const double a = 1.0 / v, b = sqrt(v);
     e0 = fmax(e0, fabs(rcp_nr(v) - a) / fabs(a));
-    e1 = fmax(e1, fabs(rsqrt_nr(v) - b) / fabs(b));
+    e1 = fmax(e1, fabs(sqrt_nr(v) - b) / fabs(b));
   }
   for (int o = 16; o > 0; o >>= 1) {
     e0 = fmax(e0, __shfl_xor_sync(0xffffffffu, e0, o));
@@ -586,14 +586,9 @@ __global__ void __launch_bounds__(QRC_THREADS) k_qr_cluster(int m, int n, int nb
     const bool works = (warp >= j && warp < w) || (warp + nwarps >= j && warp + nwarps < w);
     if (works) {
       // LAPACK's convention: beta = -sign(alpha) ||x||.  Below 2^-960 (of a column scaled to 1) the
-      // reflector is the identity.  ||x|| comes straight from rsqrt_nr's correction of q y, and signs and
-      // limits are tested on the high words: an FP64 comparison costs as much as an fma.
+      // reflector is the identity.  Signs and limits are tested on the high words: an FP64 comparison costs as much as an fma.
       const double alpha = x[r], sigma = s_sigma, aa = fabs(alpha);
-      const double qq = fma(alpha, alpha, sigma);
-      double y0;
-      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(qq));
-      const double n0 = qq * y0, e = fma(-n0, y0, 1.0);
-      const double nrm = fma(n0 * e, fma(0.375, e, 0.5), n0), tt = aa + nrm;
+      const double nrm = sqrt_nr(fma(alpha, alpha, sigma)), tt = aa + nrm;
       const bool idn = (static_cast<unsigned int>(__double2hiint(sigma)) & 0x7fffffffu) < 0x03f00000u;
       const int ahi = __double2hiint(alpha);
       const bool neg = ahi < 0 && ((ahi & 0x7fffffff) | __double2loint(alpha)) != 0;   // alpha < 0

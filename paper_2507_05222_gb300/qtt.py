@@ -545,7 +545,7 @@ def qtt_dgemm(ctx: Context, A, B, path: int = 0):
 
 
 def qtt_check_recip(ctx: Context, x):
-    """Max relative errors (reciprocal, reciprocal square root) of the QR's Newton iterations."""
+    """Max relative errors of the QR's reciprocal and square root."""
     x = np.ascontiguousarray(np.asarray(x, dtype=np.float64))
     err = np.zeros(2)
     _check(lib().qtt_check_recip(ctx.h, x.size, _dp(x), _dp(err)))

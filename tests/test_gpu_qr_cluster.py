@@ -32,3 +32,19 @@ def test_qr_cluster_edges(m, n, trans):
         Q = Q.T if trans else Q
         assert np.abs(Q - Qn).max() <= 1e-12
         assert np.abs(R / scale - Rn).max() <= 1e-12 * np.abs(Rn).max()
+
+
+def test_scalars_over_the_reflectors_range():
+    """The reciprocal and the square root that form a reflector, over what it meets: squared norms of
+    columns scaled to a largest entry in [1, 2), from 2^-960 (below it the reflector is the
+    identity) to 4 m, and the products of two norms.  Half an ulp from the last rounding, a quarter from the
+    correction's and e^3 < 2^-57 of the series: 2 ulp = 4.5e-16 with room for the product's rounding."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2507_05222_gb300 import inputs, qtt
+    g = inputs.rng(31)
+    x = np.concatenate([2.0 ** g.uniform(-960, 12, 40000), g.uniform(0.5, 4.0, 40000), np.arange(1, 1000) ** 2.0,
+                        [2.0 ** -960, 2.0 ** -959, np.nextafter(1.0, 0.0), np.nextafter(1.0, 2.0)]])
+    rcp, sqrt = qtt.qtt_check_recip(qtt.Context(0), x)
+    assert rcp <= 4.5e-16 and sqrt <= 4.5e-16
