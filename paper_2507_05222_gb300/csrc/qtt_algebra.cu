@@ -641,10 +641,9 @@ static void exact_cut(Ctx& c, CutKind kind, DBuf&& Z, int wa, int nv, const doub
   }
 }
 
-qtt_mps* apply_round_gram(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi, double eps, qtt_mps* into) {
+qtt_mps* apply_round_gram(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi, qtt_mps* into) {
   const int n = x->n, d = x->d;
   QTT_CHECK_ARG(M->n == n && M->d == d, "apply: shape mismatch");
-  QTT_CHECK_ARG(eps <= 0.0, "apply: a threshold needs the explicit product");
   std::vector<int> R(n + 1);
   for (int k = 0; k <= n; ++k) R[k] = M->bonds[k] * x->bonds[k];
   std::vector<int> mstruct = left_struct(R, d);
@@ -758,10 +757,10 @@ static int sketch_width(int chi, int d, const std::vector<int>& R) {
   return std::max(want, 1);
 }
 
-qtt_mps* apply_round_sketch(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi, double eps, qtt_mps* into) {
+qtt_mps* apply_round_sketch(Ctx& c, const qtt_mpo* M, const qtt_mps* x, int chi, qtt_mps* into) {
   const int n = x->n, d = x->d;
   QTT_CHECK_ARG(M->n == n && M->d == d, "apply: shape mismatch");
-  if (n == 1) return apply_round_gram(c, M, x, chi, eps, into);
+  if (n == 1) return apply_round_gram(c, M, x, chi, into);
   if (int64_t(d) * chi > 256)
     throw Error(QTT_ERR_UNSUPPORTED, "apply (sketched rounding): d * chi must be <= 256 (eigensolver limit)");
   std::vector<int> R(n + 1);

@@ -541,9 +541,9 @@ int mpo_apply_round(qtt_ctx* ctx, const qtt_mpo* M, const qtt_mps* x, qtt_trunc 
     std::unique_ptr<qtt_mps, void (*)(qtt_mps*)> e(mpo_mps_exact(c, M, x), free_mps);
     y.reset(round_any(c, e.get(), tr.chi_max, tr.rel_tol));
   } else if (tr.apply == QTT_APPLY_SKETCH) {
-    y.reset(apply_round_sketch(c, M, x, tr.chi_max, 0.0));
+    y.reset(apply_round_sketch(c, M, x, tr.chi_max));
   } else {
-    y.reset(apply_round_gram(c, M, x, tr.chi_max, 0.0));
+    y.reset(apply_round_gram(c, M, x, tr.chi_max));
   }
   fill_info(c, y.get(), info, &disc);
   *out = y.release();
