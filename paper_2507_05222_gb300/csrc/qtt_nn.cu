@@ -197,10 +197,10 @@ __global__ void __launch_bounds__(256) k_conv_wgrad_direct(int B, int ci, int co
   for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    s = 0.f;
-    for (int q = 0; q < 8; ++q) s += red[q];
-    grad[blk] = s;
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x & 7];
+    for (int q = 4; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if (threadIdx.x == 0) grad[blk] = s;
   }
 }
 
@@ -321,13 +321,18 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H
 constexpr size_t kWgradSmem = ((CW_TR + 2) * (CW_TC + 2) * CW_XS + CW_TR * CW_TC * CW_YS) * sizeof(float);
 static_assert(kWgradSmem >= (CW_CH * CW_CH * 9 + CW_CH) * sizeof(float), "wgrad reduction buffer");
 
-// grad[e] = sum_g part[g][e], eight lanes a value (strided over g, then a fixed tree).
+// grad[e] = sum_g part[g][e], eight lanes a value, four sums a lane (strided over g), then a fixed tree: one
+// chain of G / 8 additions a lane left gradients up to 24 % further from the 64-bit ones.
 __global__ void __launch_bounds__(256) k_conv_wsum(int64_t n, int G, const float* __restrict__ part, float* __restrict__ grad) {
   const int64_t e = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 3;
   const int l = threadIdx.x & 7;
-  float s = 0.f;
+  float s4[4] = {0.f, 0.f, 0.f, 0.f};
   if (e < n)
-    for (int g = l; g < G; g += 8) s += part[int64_t(g) * n + e];
+    for (int g = l; g < G; g += 32)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (g + 8 * q < G) s4[q] += part[int64_t(g + 8 * q) * n + e];
+  float s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
   for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (e < n && l == 0) grad[e] = s;
 }
