@@ -256,7 +256,11 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H
     }
     __syncthreads();
     if (pg < PG) {
-      for (int r = pg; r < CW_TR; r += PG) {
+      // rows of the grid only, and only the stencil's rows inside it (as in k_conv): a value that is not finite is
+      // not multiplied by the zeros outside
+      const int rows = min(CW_TR, H - i0);
+      for (int r = pg; r < rows; r += PG) {
+        const bool up = i0 + r > 0, down = i0 + r + 1 < H;
         float2 win[3][3];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -273,11 +277,14 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H
           }
           const float4 g4 = *reinterpret_cast<const float4*>(&ys[(r * CW_TC + q) * CW_YS + 4 * og]);
           const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+          if (cg == 0)
 #pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            if (cg == 0) bs[o] += g[o];
+            for (int o = 0; o < 4; ++o) bs[o] += g[o];
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
+          for (int a = 0; a < 3; ++a) {
+            if ((a == 0 && !up) || (a == 2 && !down)) continue;
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
 #pragma unroll
               for (int e = 0; e < 3; ++e) {
                 acc[o][0][3 * a + e] = fmaf(g[o], win[a][e].x, acc[o][0][3 * a + e]);

@@ -71,3 +71,39 @@ def test_weights_outside_the_grid_are_not_applied(ctx):
         good = qtt.NN(ctx, c_in, width, 3, p)
         assert net.train_step(x, y, 1e-3) == good.train_step(x, y, 1e-3)
         assert np.array_equal(net.grad(), good.grad())
+
+
+def test_values_not_finite_reach_only_the_weights_they_meet(ctx):
+    """A NaN in the grid's last row meets no upper weight (its output row would lie outside): those weights have
+    the gradient of the finite neighbours, the units that the NaN reaches being off (ReLU).  H and W are not
+    multiples of the tiles'."""
+    from paper_2507_05222_gb300 import qtt
+    c_in, width, B, H, W = 3, 12, 2, 97, 61
+    g = inputs.rng(11)
+    p = params(c_in, width, 2, 12)
+    x = g.standard_normal((B, c_in, H, W)).astype(np.float32)
+    y = g.standard_normal((B, 1, H, W)).astype(np.float32)
+    x[0, 1, H - 1, 20] = np.nan
+    x[1, 1, H - 1, 0] = np.nan
+    net = qtt.NN(ctx, c_in, width, 2, p)
+    net.train_step(x, y, 1e-3)
+    n0 = width * c_in * 9
+    dw = net.grad()[:n0].reshape(width, c_in, 3, 3)
+    pt = torch.tensor(p, dtype=torch.float64, requires_grad=True)
+    w0, b0 = pt[:n0].view(width, c_in, 3, 3), pt[n0:n0 + width]
+    w1, b1 = pt[n0 + width:-1].view(1, width, 3, 3), pt[-1:]
+
+    def conv(t, w, b):
+        t = torch.nn.functional.pad(t, (1, 1, 0, 0), mode="circular")
+        return torch.nn.functional.conv2d(torch.nn.functional.pad(t, (0, 0, 1, 1)), w, b)
+
+    xt = torch.tensor(x, dtype=torch.float64)
+    fine = torch.where(torch.isfinite(xt), xt, torch.zeros_like(xt))
+    hit = conv((~torch.isfinite(xt)).double().sum(1, keepdim=True), torch.ones(1, 1, 3, 3, dtype=torch.float64), None)
+    out = conv(torch.relu(conv(fine, w0, b0)) * (hit == 0), w1, b1)
+    loss = ((out - torch.tensor(y, dtype=torch.float64)) ** 2).mean()
+    (grad,) = torch.autograd.grad(loss, pt)
+    ref = grad[:n0].view(width, c_in, 3, 3).numpy()
+    assert np.isfinite(dw[:, 1, 0]).all()
+    assert not np.isfinite(dw[:, 1, 1:]).any()
+    assert rel(dw[:, 1, 0], ref[:, 1, 0]) < 1e-4
