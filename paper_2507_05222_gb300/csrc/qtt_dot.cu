@@ -214,11 +214,9 @@ __global__ void __launch_bounds__(DT_THREADS) k_dot_fused(const __grid_constant_
   }
 }
 
-int g_dot_cluster = -1;   // CTAs of the cluster variant (0: not available)
-
-void dot_init_attributes() {
-  if (g_dot_cluster >= 0) return;
-  g_dot_cluster = 0;
+// Whether the cluster variant is available.
+bool dot_cluster_available() {
+  bool ok = false;
   if (cudaFuncSetAttribute(k_dot_fused<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(DT_CLUSTER);
@@ -231,10 +229,10 @@ void dot_init_attributes() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k_dot_fused<true>, &cfg) == cudaSuccess && nclusters >= 1)
-      g_dot_cluster = DT_CLUSTER;
+    ok = cudaOccupancyMaxActiveClusters(&nclusters, k_dot_fused<true>, &cfg) == cudaSuccess && nclusters >= 1;
   }
   cudaGetLastError();
+  return ok;
 }
 
 }  // namespace
@@ -253,8 +251,8 @@ bool dot_fused(Ctx& c, const qtt_mps* x, const qtt_mps* y, double* out_dev) {
   for (int k = 0; k <= n; ++k) es = std::max<int64_t>(es, int64_t(x->bonds[k]) * y->bonds[k]);
   for (int k = 0; k < n; ++k)
     ts = std::max<int64_t>(ts, d * std::max<int64_t>(int64_t(y->bonds[k]) * x->bonds[k + 1], int64_t(x->bonds[k]) * y->bonds[k + 1]));
-  dot_init_attributes();
-  const bool cluster = bond <= DT_CLUSTER_BOND && g_dot_cluster > 0;
+  static const bool available = dot_cluster_available();   // once: the others of several threads wait for it
+  const bool cluster = bond <= DT_CLUSTER_BOND && available;
   DotArgs a;
   a.n = n; a.d = d;
   for (int k = 0; k <= n; ++k) { a.ab[k] = x->bonds[k]; a.bb[k] = y->bonds[k]; }
