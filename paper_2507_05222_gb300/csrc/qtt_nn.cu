@@ -30,10 +30,11 @@ unsigned nn_blocks(int64_t n, int t) { return unsigned(std::min<int64_t>((n + t 
 // the activation `act` of the layer below is not positive (its ReLU).  A CTA computes an R x 32
 // tile of pixels for 4 COT channels: a thread has four neighbouring pixels of COT channels in
 // registers, input rows and weights staged in shared memory CC input channels at a time, so that
-// 36 COT multiply-adds take 18 + 9 COT / 4 shared loads: the FP32 pipe bounds it, where one thread
+// 36 COT multiply-adds take 18 + 9 COT / 4 shared loads, where one thread
 // per output (k_conv_direct) loads an input and a weight for each multiply-add.  The order of each output's sum is
-// unchanged (input channels, then taps).  With k_conv_wgrad a training step of 8 x 128 x 128 cells,
-// width 32, depth 4 (15 GFLOP) went from 14.4 to 1.02 ms.
+// unchanged (input channels, then taps).  What bounds it is the latency of a stage's loads between its two barriers:
+// the FMA pipe is 33 to 40 % busy, the issue slots 58 to 60 %, at 2.5 warps a scheduler.  With k_conv_wgrad a training step
+// of 8 x 128 x 128 cells, width 32, depth 4 (15 GFLOP) went from 14.4 to 0.99 ms.
 template <bool FLIP>
 __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, const float* __restrict__ in,
                                               const float* __restrict__ shift, const float* __restrict__ scale,
@@ -204,6 +205,44 @@ __global__ void __launch_bounds__(256) k_conv_wgrad_direct(int B, int ci, int co
   }
 }
 
+constexpr int CW_TR = 4, CW_TC = 32, CW_CH = 32, CW_XS = 34, CW_YS = 36;   // k_conv_wgrad
+
+// One row of a tile: xr the input row above it, yr the row of dy; with TEST, the input rows above and below only where
+// they are in the grid (up, down).
+template <bool TEST>
+__device__ __forceinline__ void cw_row(const float* xr, const float* yr, bool bias, bool up, bool down, float (&acc)[4][2][9],
+                                       float (&bs)[4]) {
+  float2 win[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) win[a][e + 1] = *reinterpret_cast<const float2*>(xr + (a * (CW_TC + 2) + e) * CW_XS);
+#pragma unroll (TEST ? 1 : 4)
+  for (int q = 0; q < CW_TC; ++q) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      win[a][0] = win[a][1];
+      win[a][1] = win[a][2];
+      win[a][2] = *reinterpret_cast<const float2*>(xr + (a * (CW_TC + 2) + q + 2) * CW_XS);
+    }
+    const float4 g4 = *reinterpret_cast<const float4*>(yr + q * CW_YS);
+    const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      if (bias) bs[o] += g[o];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (TEST && ((a == 0 && !up) || (a == 2 && !down))) continue;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          acc[o][0][3 * a + e] = fmaf(g[o], win[a][e].x, acc[o][0][3 * a + e]);
+          acc[o][1][3 * a + e] = fmaf(g[o], win[a][e].y, acc[o][1][3 * a + e]);
+        }
+      }
+    }
+  }
+}
+
 // Weight and bias gradients: part[g][(o ci + c) 9 + tap] and part[g][co ci 9 + o] = the sums over the
 // pixel tiles g, g + gridDim.x, ... of dy[n, o, i, j] x'[n, c, i + a - 1, j + e - 1] (x' with the
 // layer's input affine) and of dy.  A CTA keeps a chunk of 32 x 32 channel pairs: a thread has the
@@ -211,8 +250,7 @@ __global__ void __launch_bounds__(256) k_conv_wgrad_direct(int B, int ci, int co
 // 4 x 32 tile staged in shared memory; where the layer has fewer channels the threads share the
 // tile's rows instead (pg).  The partial sums are added by k_conv_wsum in a fixed order.  (One CTA
 // per weight reads both activations from L2 for every one of the 9 co ci weights.)
-constexpr int CW_TR = 4, CW_TC = 32, CW_CH = 32, CW_XS = 34, CW_YS = 36;
-__global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H, int W, const float* __restrict__ x,
+__global__ void __launch_bounds__(256, 2) k_conv_wgrad(int B, int ci, int co, int H, int W, const float* __restrict__ x,
                                                     const float* __restrict__ shift, const float* __restrict__ scale,
                                                     const float* __restrict__ dy, float* __restrict__ part) {
   extern __shared__ __align__(16) float cw_sm[];
@@ -235,6 +273,7 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int n = t / (tw * th), i0 = ((t / tw) % th) * CW_TR, j0 = (t % tw) * CW_TC;
     __syncthreads();
+    int top = 0;                                              // largest magnitude staged, as an integer
     for (int e = tid; e < CW_CH * (CW_TR + 2) * (CW_TC + 2); e += 256) {
       const int q = e % (CW_TC + 2), r = (e / (CW_TC + 2)) % (CW_TR + 2), c = e / ((CW_TC + 2) * (CW_TR + 2));
       const int ii = i0 + r - 1;
@@ -247,51 +286,24 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(int B, int ci, int co, int H
         if (shift) v = (v - shift[c0 + c]) * scale[c0 + c];
       }
       xs[(r * (CW_TC + 2) + q) * CW_XS + c] = v;
+      top = max(top, __float_as_int(v) & 0x7fffffff);
     }
     for (int e = tid; e < CW_CH * CW_TR * CW_TC; e += 256) {
       const int q = e % CW_TC, r = (e / CW_TC) % CW_TR, o = e / (CW_TC * CW_TR);
       const int ii = i0 + r, jj = j0 + q;
-      ys[(r * CW_TC + q) * CW_YS + o] =
-          (o < no && ii < H && jj < W) ? dy[(int64_t(n) * co + o0 + o) * per + int64_t(ii) * W + jj] : 0.f;
+      const float v = (o < no && ii < H && jj < W) ? dy[(int64_t(n) * co + o0 + o) * per + int64_t(ii) * W + jj] : 0.f;
+      ys[(r * CW_TC + q) * CW_YS + o] = v;
+      top = max(top, __float_as_int(v) & 0x7fffffff);
     }
-    __syncthreads();
+    // Rows outside the grid count as zeros, which a value that is not finite must not meet (they are no part of the
+    // sums): a tile with such a value takes its rows with the test, which in every tile cost 9 us of a 104 us step.
+    const bool finite = __syncthreads_or(top >= 0x7f800000) == 0;
     if (pg < PG) {
-      // rows of the grid only, and only the stencil's rows inside it (as in k_conv): a value that is not finite is
-      // not multiplied by the zeros outside
-      const int rows = min(CW_TR, H - i0);
-      for (int r = pg; r < rows; r += PG) {
-        const bool up = i0 + r > 0, down = i0 + r + 1 < H;
-        float2 win[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-          for (int e = 0; e < 2; ++e)
-            win[a][e + 1] = *reinterpret_cast<const float2*>(&xs[((r + a) * (CW_TC + 2) + e) * CW_XS + 2 * cg]);
-#pragma unroll 4
-        for (int q = 0; q < CW_TC; ++q) {
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            win[a][0] = win[a][1];
-            win[a][1] = win[a][2];
-            win[a][2] = *reinterpret_cast<const float2*>(&xs[((r + a) * (CW_TC + 2) + q + 2) * CW_XS + 2 * cg]);
-          }
-          const float4 g4 = *reinterpret_cast<const float4*>(&ys[(r * CW_TC + q) * CW_YS + 4 * og]);
-          const float g[4] = {g4.x, g4.y, g4.z, g4.w};
-          if (cg == 0)
-#pragma unroll
-            for (int o = 0; o < 4; ++o) bs[o] += g[o];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            if ((a == 0 && !up) || (a == 2 && !down)) continue;
-#pragma unroll
-            for (int o = 0; o < 4; ++o)
-#pragma unroll
-              for (int e = 0; e < 3; ++e) {
-                acc[o][0][3 * a + e] = fmaf(g[o], win[a][e].x, acc[o][0][3 * a + e]);
-                acc[o][1][3 * a + e] = fmaf(g[o], win[a][e].y, acc[o][1][3 * a + e]);
-              }
-          }
-        }
+      for (int r = pg; r < (finite ? CW_TR : min(CW_TR, H - i0)); r += PG) {
+        const float* xr = xs + r * (CW_TC + 2) * CW_XS + 2 * cg;
+        const float* yr = ys + r * CW_TC * CW_YS + 4 * og;
+        if (finite) cw_row<false>(xr, yr, cg == 0, true, true, acc, bs);
+        else cw_row<true>(xr, yr, cg == 0, i0 + r > 0, i0 + r + 1 < H, acc, bs);
       }
     }
   }
