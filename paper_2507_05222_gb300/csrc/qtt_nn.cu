@@ -346,11 +346,16 @@ __global__ void __launch_bounds__(256) k_conv_wsum(int64_t n, int G, const float
   const int64_t e = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 3;
   const int l = threadIdx.x & 7;
   float s4[4] = {0.f, 0.f, 0.f, 0.f};
-  if (e < n)
-    for (int g = l; g < G; g += 32)
+  if (e < n) {
+    int g = l;
+#pragma unroll 2
+    for (; g + 24 < G; g += 32)
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (g + 8 * q < G) s4[q] += part[int64_t(g + 8 * q) * n + e];
+      for (int q = 0; q < 4; ++q) s4[q] += part[int64_t(g + 8 * q) * n + e];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (g + 8 * q < G) s4[q] += part[int64_t(g + 8 * q) * n + e];
+  }
   float s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
   for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (e < n && l == 0) grad[e] = s;
