@@ -436,10 +436,10 @@ static void top_vectors_as_core(Ctx& c, const double* V, int nv, int b, double* 
 //   CUT_LEFT   b = m:  Q^T of (T Z)^T = Q R, T the explicit left unfolding of m rows (anchored at the
 //              last bond that left_struct takes whole), P = Z Q;
 //   CUT_TRUNC  otherwise: the top eigenvectors of the cut's density matrix.
-// At chi = 64 and 2^20 cells 7 of the 19 cuts truncate, at a grid's full rank none.  Measured on a
-// GB300: a full-rank product at 2^10 cells 8.5 -> 0.40 ms, at 2^13 cells 14.3 -> 0.95 ms, a sum of
-// two trains of bond 24 at the bond 48 of the exact result (2^20 cells) 28.1 -> 2.5 ms, the
-// sketched product at 2^20 cells and chi = 64 76.7 -> 49.5 ms.
+// At chi = 64 and 2^20 cells 7 of the 19 cuts truncate, at a grid's full rank none.  On a GB300, with an eigenproblem
+// at every cut and now (the QR and the eigensolver have changed as well since): a full-rank product at 2^10 cells
+// 8.2 -> 0.38 ms, at 2^13 cells 14.0 -> 0.73 ms, a sum of two trains of bond 24 at the bond 48 of the exact result
+// (2^20 cells) 27.9 -> 1.67 ms, the sketched product at 2^20 cells and chi = 64 76.7 -> 19.9 ms (49.5 by this rule alone).
 // Only for rel_tol = 0: a threshold needs the singular values of every cut.
 enum CutKind { CUT_RIGHT, CUT_BOND, CUT_LEFT, CUT_TRUNC };
 static CutKind cut_kind(int b, int nv, int a, int m) {

@@ -10,7 +10,8 @@
 // pivot floor; the vectors below it (the next level's, or null vectors) are a Householder basis of the
 // orthogonal complement.
 // Refinement (k_psd_refine): Newton-Schulz and Ogita-Aishima iterations (Ogita and Aishima, Japan
-// J. Indust. Appl. Math. 35, 2018) until the next correction across the cut would be below rounding,
+// J. Indust. Appl. Math. 35, 2018) until the next correction across the cut would be below rounding (at
+// most eight; all eight where the cut lies among eigenvalues of pure rounding, whose corrections do not shrink),
 // products of 8 x 8 tiles dealt to the CTAs, grid
 // barriers (bounded, as in qtt_cg.cu) between them.  With a factor F (S = F^T F) X^T S X is formed
 // as (F X)^T (F X), which keeps the tail on its own scale, and levels follow down to 1e-24.
@@ -912,8 +913,9 @@ void eigh_psd_init_attributes() {
   g_psd_per_sm = per_sm;
 }
 
-// Orders 2 to 128, where the start's matrix fits a CTA's shared memory.  Against the general solver: a sketched
-// product at 20 bits (bond 64) 49.5 -> 23.5 ms, the encoding of 2^20 values 12.7 -> 3.2 ms; error against the
+// Orders 2 to 128, where the start's matrix fits a CTA's shared memory.  Against the general solver, when this one came
+// in (everything else the same): a sketched product at 20 bits (bond 64) 49.5 -> 23.5 ms, the encoding of 2^20 values
+// 12.7 -> 3.2 ms; with the present QR 19.9 and 2.9 ms.  Rank 5 of 32 kept at order 64: 2.99 -> 0.46 ms.  Error against the
 // exact decomposition of the same product 4e-13 .. 3e-11 -> 2e-13 (12 inputs).
 bool eigh_psd_fits(int n, int m) {
   eigh_psd_init_attributes();

@@ -34,7 +34,7 @@ unsigned nn_blocks(int64_t n, int t) { return unsigned(std::min<int64_t>((n + t 
 // per output (k_conv_direct) loads an input and a weight for each multiply-add.  The order of each output's sum is
 // unchanged (input channels, then taps).  What bounds it is the latency of a stage's loads between its two barriers:
 // the FMA pipe is 33 to 40 % busy, the issue slots 58 to 60 %, at 2.5 warps a scheduler.  With k_conv_wgrad a training step
-// of 8 x 128 x 128 cells, width 32, depth 4 (15 GFLOP) went from 14.4 to 0.99 ms.
+// of 8 x 128 x 128 cells, width 32, depth 4 (15 GFLOP) went from 14.4 to 0.97 ms.
 template <bool FLIP>
 __global__ void __launch_bounds__(256) k_conv(int ni, int no, int H, int W, const float* __restrict__ in,
                                               const float* __restrict__ shift, const float* __restrict__ scale,
